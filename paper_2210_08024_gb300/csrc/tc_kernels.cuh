@@ -18,6 +18,7 @@
 #pragma once
 #include <type_traits>
 
+#include "tc_dual.cuh"
 #include "tc_mlp.cuh"
 #include "tc_mlp_mma.cuh"
 #include "tc_phys.cuh"
@@ -373,8 +374,7 @@ constexpr double JAC_REUSE = 1e-3;
 template <int LPC = 1>
 TCG_FN int newton_iter(const CellC<double>& c, const DevParams& p, double mu, double Kinv, const double* yn,
                        double dts, double* y, double& xe_g, double& td_g, double (*Jk)[3], bool reuse,
-                       double& rel, bool& full, Equil<double>* qb,
-                       const ChemT<double>* b0 = nullptr, const CoolT<double>* k0 = nullptr) {
+                       double& rel, bool& full, Equil<double>* qb) {
   double f0[3], J[3][3];
   if constexpr (LPC == 4) {
     if (reuse) {
@@ -427,20 +427,11 @@ TCG_FN int newton_iter(const CellC<double>& c, const DevParams& p, double mu, do
     // then the T_mu column from the base point's temperature blocks stepped to T + dT
     // (temp_blocks_step).  The columns start their C/O/e and dust-temperature solves from the base
     // point's roots, ~1e-7 away, and take one Newton step of the C/O/e balance
-    // (converged to ~1e-14 from there; the loop would take a second to confirm it).  The
-    // temperature blocks at the base point are given by the caller at a substep's first
-    // iteration (the substep start's, the same temperature), else built here.
+    // (converged to ~1e-14 from there; the loop would take a second to confirm it).
     if (reuse) TCG_COUNT_D(chord64_it);
     else TCG_COUNT_D(newton64_it);
-    ChemT<double> b;
-    CoolT<double> k;
-    if (b0) {
-      b = *b0;
-      k = *k0;
-    } else {
-      b = chem_T(c, mu * y[0], p.flags);
-      k = cool_T(c, b, p.flags);
-    }
+    ChemT<double> b = chem_T(c, mu * y[0], p.flags);
+    CoolT<double> k = cool_T(c, b, p.flags);
     feval64(c, b, k, y[1], y[2], Kinv, xe_g, td_g, f0, qb);
     if (reuse) {
       for (int i = 0; i < 3; ++i)
@@ -494,8 +485,7 @@ TCG_FN int newton_iter(const CellC<double>& c, const DevParams& p, double mu, do
 template <int LPC = 1>
 TCG_FN int newton_solve(const CellC<double>& c, const DevParams& p, double mu, double Kinv, const double* yn,
                         double dts, double* y, double& xe_g, double& td_g, int maxit = 0,
-                        Equil<double>* qb = nullptr, int* spent = nullptr,
-                        const ChemT<double>* b0 = nullptr, const CoolT<double>* k0 = nullptr) {
+                        Equil<double>* qb = nullptr, int* spent = nullptr) {
   const int nmax = (maxit > 0) ? maxit : p.newton_max;
   double Jk[3][3];
   bool reuse = false;
@@ -503,8 +493,7 @@ TCG_FN int newton_solve(const CellC<double>& c, const DevParams& p, double mu, d
   for (int it = 1; it <= nmax; ++it) {
     double rel;
     bool full;
-    const int r = newton_iter<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, Jk, reuse, rel, full, qb,
-                                   (it == 1) ? b0 : nullptr, (it == 1) ? k0 : nullptr);
+    const int r = newton_iter<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, Jk, reuse, rel, full, qb);
     if (spent) *spent = it;
     if (r < 0) return -1;
     if (r > 0) return it;
@@ -518,11 +507,10 @@ TCG_FN int newton_solve(const CellC<double>& c, const DevParams& p, double mu, d
 // with the dust temperature solved; gives the substep length of Sec. 6.1.
 template <class F>
 TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneState& s, F& td_g, double& H0,
-                          double& CH2, double& CHp, ChemT<F>* bo = nullptr, CoolT<F>* ko = nullptr) {
+                          double& CH2, double& CHp) {
   const double T = s.mu * s.Tmu;
   ChemT<F> b = chem_T(cf, to_prec<F>(T), p.flags);
   CoolT<F> k = cool_T(cf, b, p.flags);
-  if (bo) { *bo = b; *ko = k; }
   Equil<F> q;
   q.xe = to_prec<F>(s.xe); q.xCp = to_prec<F>(s.xCp); q.xCO = to_prec<F>(s.xCO);
   q.xOp = cf.xOtot * to_prec<F>(s.xHp);
@@ -536,6 +524,114 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
   H0 = n * double(sr.G) - n * n * double(sr.L);
   CH2 = double(sr.form) - double(sr.dest);
   CHp = double(sr.ion) - double(sr.rec);
+}
+
+// Newton with the Jacobian from FP32 dual numbers (source_tangents): the fast path of
+// the FP64 solve.  Each iteration evaluates f once, in FP64, where the forward
+// differences of newton_iter take three more evaluations; the first iteration takes f
+// from the substep start's source terms `src` = (H, C_H2, C_H+), so it evaluates nothing
+// (they hold the stored x_e instead of the one at the new mu: the start of the iteration
+// is that much off, its root is not).  The FP32 Jacobian is good to ~1e-6, so steps
+// contract quadratically until there and by ~1e-6 a step from there on.
+//
+// Converged when every step is below rtol |y_i| as in newton_iter, or one step earlier,
+// when two steps in a row show that the next would lie far below it: with rho = d_k /
+// d_(k-1), what remains after step k is at most ~rho d_k, accepted below 1e-2 rtol
+// (measured on 20,000 slab cells against a 64-bit reference converged to rounding: 2-norm
+// error of T 1.4e-16, of x_e 2.3e-16; the plain iteration 3.9e-15 and 4.7e-14).  The C/O/e equilibrium
+// of the last evaluation is moved along the last step by its derivatives, which leaves
+// less than the step squared (below 1e-16).
+//
+// Returns the iterations, or -1 when a step would have to be damped, fails to shrink by
+// half after the second iteration or is not finite, or when TAN_MAXIT iterations pass;
+// the plain solver then takes the substep from its start, as if this one had not been
+// tried.  Hard substeps (2% of the random states'
+// iterations, 0.04% of the slab's) thus keep the plain iteration's path, with its damping,
+// predictor and halving decisions.  (Damping here too solved some substeps that the plain
+// iteration halves, which changed the substep grid of 5 in 13,824 cells near x_H = 0.)
+constexpr int TAN_MAXIT = 12;
+constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
+TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double mu, double Kinv,
+                          const double* yn, double dts, const double* src, double* y, double& xe_g, double& td_g,
+                          Equil<double>* qb) {
+  double f[3] = {src[0] * Kinv, src[1], src[2]};
+  const float hk = float(1.0 / (double(c.muH) * KB * 1.5));
+  float prev = -1.0f;  // size of the previous step, if that was whole
+  const int maxit = (p.newton_max < TAN_MAXIT) ? p.newton_max : TAN_MAXIT;
+  for (int it = 1; it <= maxit; ++it) {
+    TCG_COUNT_D(tangent_it);
+    if (it > 1) {
+      ChemT<double> b = chem_T(c, mu * y[0], p.flags);
+      CoolT<double> k = cool_T(c, b, p.flags);
+      feval64(c, b, k, y[1], y[2], Kinv, xe_g, td_g, f, qb);
+    }
+    const double xH = 1.0 - 2.0 * y[1] - y[2];
+    const float y0 = float(y[0]), x2 = float(y[1]), xp = float(y[2]);
+    float df[3][3], dq[3][3];
+    source_tangents(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), df, dq);
+    // rows scaled: (T_mu equation / T_mu, x_H2, x_H+); unknowns (ln T_mu, x_H2, x_H+)
+    const float iy0 = 1.0f / y0, h = float(dts);
+    float J[3][3], r[3], u[3];
+    double d[3], rhs[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      rhs[i] = -(y[i] - yn[i] - dts * f[i]);
+      const float s = (i == 0) ? iy0 : 1.0f;
+      r[i] = float(rhs[i]) * s;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) J[i][j] = ((i == j) ? 1.0f : 0.0f) - (h * s) * df[i][j];
+      // an abundance near or below FP32's range matters to nothing but itself: its row
+      // decouples and its step is taken in FP64
+      if (i > 0 && y[i] < TAN_TRACE) {
+        d[i] = rhs[i] / double(J[i][i]);
+        r[i] = 0.0f;
+        J[i][0] = J[i][3 - i] = 0.0f;
+      }
+    }
+    if (!solve3<float>(J, r, u)) return -1;
+    // T_mu, x_H2, x_H+ and x_H must keep 2% of their values (damped_step limits at 1%),
+    // except an abundance whose step is below 1e-8 (too little to matter to the others): it
+    // may fall to any positive value, and to 1% of its value where the step rounds to less
+    bool whole = true;
+    float rel = fabsf(u[0]);
+    d[0] = double(u[0]) * y[0];
+#pragma unroll
+    for (int i = 1; i < 3; ++i) {
+      const bool trace = y[i] < TAN_TRACE;
+      if (trace) u[i] = float(d[i]);
+      else d[i] = double(u[i]);
+      const float x = (i == 1) ? x2 : xp;
+      if (fabsf(u[i]) <= 1e-8f) {
+        if (!(y[i] + d[i] > 0.0) && d[i] != 0.0) {
+          d[i] = -0.99 * y[i];
+          whole = false;
+        }
+      } else if (!(u[i] >= -0.98f * x)) {
+        return -1;
+      }
+      const double yi = y[i] + d[i];
+      const float ri = trace ? float(fabs(d[i]) / (fabs(yi) + 1e-300)) : fabsf(u[i]) / (fabsf(float(yi)) + 1e-30f);
+      rel = fmaxf(rel, ri);
+    }
+    if (!(u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * float(xH)) || !isfinite(rel)) return -1;
+    y[0] += d[0]; y[1] += d[1]; y[2] += d[2];
+    if (!whole) {
+      prev = -1.0f;
+      continue;
+    }
+    const float rtol = float(p.rtol);
+    if (it > 1 && (rel <= rtol || (prev > 0.0f && rel < 1e-2f * prev && rel * (rel / prev) <= 1e-2f * rtol))) {
+      // u is at most ~1e-6 here: the change of x_e, x_C+ and x_CO to first order
+      qb->xe += double(dq[0][0] * u[0] + dq[0][1] * u[1] + dq[0][2] * u[2]);
+      qb->xCp += double(dq[1][0] * u[0] + dq[1][1] * u[1] + dq[1][2] * u[2]);
+      qb->xCO += double(dq[2][0] * u[0] + dq[2][1] * u[1] + dq[2][2] * u[2]);
+      xe_g = qb->xe;
+      return it;
+    }
+    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev)) return -1;
+    prev = rel;
+  }
+  return -1;
 }
 
 // Accepts the substep's root y: applies the temperature floor, re-solves the C/O/e
@@ -638,10 +734,9 @@ constexpr int RESCUE_ITER_FACTOR = 8;
 // solve, or -1.
 template <int LPC = 1>
 TCG_FN int solve_from_start64(const CellC<double>& c, const DevParams& p, double mu, double Kinv, const double* yn,
-                              double dts, double* y, double& xe_g, double& td_g, int& status, Equil<double>* qb,
-                              const ChemT<double>* b0 = nullptr, const CoolT<double>* k0 = nullptr) {
+                              double dts, double* y, double& xe_g, double& td_g, int& status, Equil<double>* qb) {
   y[0] = yn[0]; y[1] = yn[1]; y[2] = yn[2];
-  int it = newton_solve<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, 0, qb, nullptr, b0, k0);
+  int it = newton_solve<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, 0, qb);
   if (it >= 0) return it;
   status |= ST_PREDICTOR;
   picard_predictor(c, p, mu, Kinv, yn, dts, y, xe_g, td_g);
@@ -766,13 +861,13 @@ TCG_FN int chord64_from_seed(const CellC<double>& c, const CellC<float>& cf, con
 
 // Solves one substep of length dts by the FP64 Newton iteration, from `seed` when
 // given (the root is the same; a seeded solve that fails is retried from the start
-// state), else from the start state, then from the predictor; a substep that fails
-// from both is retried at half length (up to 30 times) and the cell flagged ST_NEWTON.
+// state), else from the start state (with `src`, the start's source terms, first by
+// newton_tangent), then from the predictor; a substep that fails from both is retried
+// at half length (up to 30 times) and the cell flagged ST_NEWTON.
 template <int LPC = 1>
 TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double dt, double dts, bool last,
                             LaneState& s, double& xe_g, double& td_g, const double* seed = nullptr,
-                            const CellC<float>* cf = nullptr,
-                            const ChemT<double>* b0 = nullptr, const CoolT<double>* k0 = nullptr) {
+                            const CellC<float>* cf = nullptr, const double* src = nullptr) {
   const double yn[3] = {s.Tmu, s.xH2, s.xHp};
   const double Kinv = 1.0 / c.K;
   double y[3] = {yn[0], yn[1], yn[2]};
@@ -793,15 +888,19 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
       s.status |= ST_SEED_FAIL;
     }
   }
-  // b0, k0: the temperature blocks at the start state, if the caller has them
-  if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb, b0, k0);
+  if (src) {
+    double xg = xe_g, tg = td_g;
+    it = newton_tangent(c, *cf, p, s.mu, Kinv, yn, dts, src, y, xg, tg, &qb);
+    if (it >= 0) { xe_g = xg; td_g = tg; }
+  }
+  if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);
   int halv = 0;
   while (it < 0 && halv < 30) {
     s.status |= ST_NEWTON;
     dts *= 0.5;
     last = false;
     ++halv;
-    it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb, b0, k0);
+    it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);
   }
   if (it < 0) {
     s.status |= ST_NONFIN;
@@ -817,33 +916,30 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
 // factor.  `src`, when given, receives those terms (H, C_H2, C_H+).
 template <class F>
 TCG_FN double substep_start_t(const CellC<F>& cc, double K, const DevParams& p, double dt, const LaneState& s,
-                              F& td_g, bool& last, double* src = nullptr, ChemT<F>* bo = nullptr,
-                              CoolT<F>* ko = nullptr) {
+                              F& td_g, bool& last, double* src = nullptr) {
   double H0, CH2, CHp;
-  start_sources<F>(cc, p, s, td_g, H0, CH2, CHp, bo, ko);
+  start_sources<F>(cc, p, s, td_g, H0, CH2, CHp);
   if (src) { src[0] = H0; src[1] = CH2; src[2] = CHp; }
   return substep_len(p, dt - s.t, K * s.Tmu, H0, CH2, CHp, last);
 }
 TCG_FN double substep_start64(const CellC<double>& c, const DevParams& p, double dt, const LaneState& s,
-                              double& td_g, bool& last, double* src = nullptr, ChemT<double>* bo = nullptr,
-                              CoolT<double>* ko = nullptr) {
-  return substep_start_t<double>(c, c.K, p, dt, s, td_g, last, src, bo, ko);
+                              double& td_g, bool& last, double* src = nullptr) {
+  return substep_start_t<double>(c, c.K, p, dt, s, td_g, last, src);
 }
 
+// One substep of mode 1; cf is the FP32 copy of the cell's constants.
+template <int LPC = 1>
+TCG_FN void substep_newton64(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double dt, LaneState& s,
+                             double& xe_g, double& td_g) {
+  bool last;
+  double src[3];
+  const double dts = substep_start64(c, p, dt, s, td_g, last, src);
+  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, src);
+}
 template <int LPC = 1>
 TCG_FN void substep_newton64(const CellC<double>& c, const DevParams& p, double dt, LaneState& s, double& xe_g,
                              double& td_g) {
-  bool last;
-  if constexpr (LPC == 1) {
-    // the start's temperature blocks serve the first Newton iteration (same T)
-    ChemT<double> b0;
-    CoolT<double> k0;
-    const double dts = substep_start64(c, p, dt, s, td_g, last, nullptr, &b0, &k0);
-    solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, nullptr, &b0, &k0);
-  } else {
-    const double dts = substep_start64(c, p, dt, s, td_g, last);
-    solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g);
-  }
+  substep_newton64<LPC>(c, cast_cell<float>(c), p, dt, s, xe_g, td_g);
 }
 
 // ------------------------------------------------------------------ mode 2: mixed precision
@@ -1149,13 +1245,12 @@ TCG_FN bool seed_from_outputs(const float* o, const double* g, const LaneState& 
 //   3 blocks (168 registers, compiler's choice) 546 / 403
 //   4 blocks (128) 394 / 195,  5 (96) 375 / 174,  6 (80) 365 / 164,
 //   7 (72) 362 / 156,  8 (64) 363 / 152.
-// With the FP64 exp and log out of line (a shorter per-thread stack) the autotuner picks
-// 4 resident blocks of 128 for FP64 Newton and the paper scheme, and their kernels are
-// compiled for 6 (80 registers): FP64 Newton 214.6 -> 212.9 ms, paper scheme 50.9 ->
-// 50.0 (4 blocks: 214.1 / 50.7, 5: 213.3 / 50.3).  The seeded FP64 kernel keeps 8
-// (293.5 ms; 300.1 at 6).
+// The paper scheme is compiled for 6 (80 registers; 4 blocks: 50.7 ms, 5: 50.3, 6: 50.0 when
+// its FP64 exp and log went out of line), the FP64 Newton kernels for 8: with the Jacobian
+// from dual numbers, FP32 work that overlaps the FP64 pipe, 4 / 5 / 6 / 8 blocks took
+// 96.1 / 93.4 / 90.7 / 87.6 ms.  The seeded FP64 kernel keeps 8 (293.5 ms; 300.1 at 6).
 constexpr int STEP_MIN_BLOCKS = 8;
-constexpr int STEP_MIN_BLOCKS_FP64 = 6;
+constexpr int STEP_MIN_BLOCKS_PAPER = 6;
 // The warp-cooperative kernels (four lanes per cell) serve launches too small to fill
 // the GPU, where the time is the latency of the slowest cells: 4 resident blocks (128
 // registers per thread) spill less.
@@ -1170,8 +1265,8 @@ constexpr int STEP_MIN_BLOCKS_MIXED = 12;
 
 template <int MODE, bool BATCH, int LPC = 1>
 __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? STEP_MIN_BLOCKS_MIXED
-                                                      : (MODE == 0 || MODE == 1) ? STEP_MIN_BLOCKS_FP64
-                                                                              : STEP_MIN_BLOCKS)
+                                                      : (MODE == 0) ? STEP_MIN_BLOCKS_PAPER
+                                                                    : STEP_MIN_BLOCKS)
                                                   : STEP_MIN_BLOCKS_COOP)
     k_step(DevFields f1, const BoxTable* __restrict__ boxes, DevParams p, double dt, unsigned long long* cursor,
            long long ntotal, const MlpDev* __restrict__ mlp) {
@@ -1182,7 +1277,7 @@ __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? 
   float lf[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   LaneState s;
   CellC<double> c;
-  CellC<float> cf;   // FP32 copy of the cell constants (mixed and seeded modes)
+  CellC<float> cf;   // FP32 copy of the cell constants (all modes but the paper's scheme)
   CellC<df64> cd;    // df64 copy (mixed modes: substep-start sources and polish)
   double xe_g = -1.0, td_g = -1.0;
   float xe_gf = -1.f, td_gf = -1.f;
@@ -1235,8 +1330,8 @@ __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? 
           xe_g = q0.xe;
           td_g = -1.0;
         }
+        if constexpr (MODE != 0) cf = cast_cell<float>(c);
         if constexpr (MIXED || SEEDED) {
-          cf = cast_cell<float>(c);
           xe_gf = float(s.xe);
           td_gf = -1.f;
         }
@@ -1296,7 +1391,7 @@ __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? 
         } else if constexpr (MODE == 0) {
           substep_paper(c, p, dt, s);
         } else if constexpr (MODE == 1) {
-          substep_newton64<LPC>(c, p, dt, s, xe_g, td_g);
+          substep_newton64<LPC>(c, cf, p, dt, s, xe_g, td_g);
         } else if constexpr (MODE == 2) {
           substep_mixed<LPC>(c, cd, cf, p, dt, s, xe_gf, td_gf, td_hp);
         }

@@ -8,8 +8,10 @@
 //   CoolT<F>   temperature-only pieces of the heating and cooling functions.
 // Powers of T and psi are taken as exp(c ln T), exp(c ln psi) from one logarithm.
 //
-// F is double for the FP64 paths, float for the mixed path's Newton iterations and df64
-// (double-float, tc_df64.cuh) for its high-precision evaluations.  Terms
+// F is double for the FP64 paths, float for the mixed path's Newton iterations, df64
+// (double-float, tc_df64.cuh) for its high-precision evaluations and dualf (FP32 dual
+// numbers, tc_dual.cuh) for the derivatives of the FP64 Newton's Jacobian, which takes
+// its cell constants in FP32 (type FC, elsewhere the same as F).  Terms
 // the paper names but does not print (closures: cited fits and tables it does not
 // reproduce) use one stated definition each, labelled where it is a stand-in for the
 // cited source; the CPU checker uses the same definitions, written independently.
@@ -35,12 +37,16 @@
 #endif
 // Work-counting hooks: empty in the library; the host work counter (tc_workcount.cu)
 // defines them to count calls and inner iterations of the step's building blocks.
-// TCG_COUNT is used inside templates on the scalar type F; TCG_COUNT_D in FP64 code.
+// TCG_COUNT is used inside templates on the scalar type F; TCG_COUNT_D in FP64 code;
+// TCG_COUNT_T names the type.
 #ifndef TCG_COUNT
 #define TCG_COUNT(name)
 #endif
 #ifndef TCG_COUNT_D
 #define TCG_COUNT_D(name)
+#endif
+#ifndef TCG_COUNT_T
+#define TCG_COUNT_T(name, type)
 #endif
 
 namespace tcg {
@@ -247,14 +253,14 @@ template <class F> struct ChemT {
 // Electrons of hot gas at log10 T = lt: x_e,He,CIE (two logistic steps, at 4.45 and
 // 4.95, whose exponentials differ by the constant factor exp(0.5/0.06)) + Z'_g
 // x_e,metal,CIE (one step at 5.5).
-template <class F> TCG_FN F xe_hot_of(const CellC<F>& c, F lt) {
+template <class F, class FC> TCG_FN F xe_hot_of(const CellC<FC>& c, F lt) {
   F eHe = m_exp((F(4.45) - lt) * F(1.0 / 0.06));
   F xeHe = F(0.1) * (F(1) / (F(1) + eHe) + F(1) / (F(1) + eHe * F(4160.262005375057)));  // exp(25/3)
   F xeMet = F(0.012) * logistic((lt - F(5.5)) * F(4));
   return xeHe + c.Zg * xeMet;
 }
 
-template <class F> TCG_BIG ChemT<F> chem_T(const CellC<F>& c, F T, unsigned flags) {
+template <class F, class FC> TCG_BIG ChemT<F> chem_T(const CellC<FC>& c, F T, unsigned flags) {
   TCG_COUNT(chem_T);
   ChemT<F> b;
   b.T = T;
@@ -325,13 +331,13 @@ template <class F> TCG_FN F rovib_lte_of(F lT3, F iT3) {
   return Lrot + Lvib;
 }
 // CIE cooling of He and metals (before the S weighting) at log10 T = lt
-template <class F> TCG_FN F cie_of(const CellC<F>& c, F lt) {
+template <class F, class FC> TCG_FN F cie_of(const CellC<FC>& c, F lt) {
   F z1 = (lt - F(5.0)) * F(1.0 / 0.15), z2 = (lt - F(5.35)) * F(1.0 / 0.28), z3 = (lt - F(6.3)) * F(1.0 / 0.35);
   return F(2.0e-23) * m_exp(F(-0.5) * z1 * z1) +
          c.Zg * (F(5.4e-22) * m_exp(F(-0.5) * z2 * z2) + F(5.0e-23) * m_exp(F(-0.5) * z3 * z3));
 }
 
-template <class F> TCG_BIG CoolT<F> cool_T(const CellC<F>& c, const ChemT<F>& b, unsigned flags) {
+template <class F, class FC> TCG_BIG CoolT<F> cool_T(const CellC<FC>& c, const ChemT<F>& b, unsigned flags) {
   TCG_COUNT(cool_T);
   CoolT<F> k;
   const F T = b.T, lnT = b.lnT;
@@ -634,7 +640,7 @@ template <class F> struct HRate {
 // xH is the atomic fraction 1 - 2 x_H2 - x_H+ (Sec. 3.1.3), passed in so that the
 // mixed-precision path can form it in FP64 and hand the FP32 rates an accurate value
 // when x_H+ -> 1 or x_H2 -> 1/2.
-template <class F> TCG_FN HRate<F> h_rates(const CellC<F>& c, const ChemT<F>& b, F xH2, F xH,
+template <class F, class FC> TCG_FN HRate<F> h_rates(const CellC<FC>& c, const ChemT<F>& b, F xH2, F xH,
                                                                F xe, F lpsi) {
   HRate<F> r;
   F zcrH2 = F(2) * c.xi * (F(2.3) * xH2 + F(1.5) * xH);        // Eq. eq:H2_cr
@@ -649,7 +655,7 @@ template <class F> TCG_FN HRate<F> h_rates(const CellC<F>& c, const ChemT<F>& b,
   return r;
 }
 
-template <class F> TCG_FN F log_psi(const CellC<F>& c, const ChemT<F>& b, F xe) {
+template <class F, class FC> TCG_FN F log_psi(const CellC<FC>& c, const ChemT<F>& b, F xe) {
   return m_log(c.G0 * b.sqT / m_max(xe * c.n, F(1e-30)) + F(50));
 }
 
@@ -666,7 +672,7 @@ template <class F> struct Src {
 // Heating (Eq. e:heating) and cooling (Eq. eq:cooling_fnct) at (T, x_H2, x_H+, q) with
 // the atomic fraction xH given.  Td_fixed > 0 freezes the dust temperature; otherwise it
 // is solved from Td_guess.
-template <class F> TCG_BIG Src<F> source(const CellC<F>& c, const ChemT<F>& b, const CoolT<F>& k,
+template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const ChemT<F>& b, const CoolT<F>& k,
                                                             F xH2, F xHp, F xH, const Equil<F>& q, F Td_fixed,
                                                             F Td_guess) {
   TCG_COUNT(source);
@@ -752,7 +758,8 @@ template <class F> TCG_BIG Src<F> source(const CellC<F>& c, const ChemT<F>& b, c
     F ne2 = xe * n * F(0.01);
     Lmet += c.Zg * xe * xHp * k.nebT / (F(1) + F(0.12) * m_exp(k.nebX * m_log(ne2)));
     // gas-dust (Eq. eq:gas-dust)
-    s.Td = (Td_fixed > F(0)) ? Td_fixed : dust_T(c, b.T, b.sqT, Td_guess);
+    if constexpr (Prec<F>::cls == 3) s.Td = Td_fixed;  // derivatives: the caller has differentiated the root
+    else s.Td = (Td_fixed > F(0)) ? Td_fixed : dust_T(c, b.T, b.sqT, Td_guess);
     Lmet += F(3.2e-34) * b.sqT * (b.T - s.Td) * c.Zd;
   }
   F L = Lhyd + (F(1) - b.S) * Lmet + b.S * k.cie;

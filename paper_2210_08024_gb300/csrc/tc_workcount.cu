@@ -23,17 +23,19 @@
 namespace wc {
 struct Calls {
   long long chem_T, cool_T, temp_step, equil, equil_it, dust, dust_it, source;
-  long long newton64_it, chord64_it, newton32_it, polish_it, substep_paper, picard_it;
+  long long newton64_it, chord64_it, tangent_it, newton32_it, polish_it, substep_paper, picard_it;
 };
-Calls calls[3];  // [0] FP64, [1] FP32, [2] df64 (double-float)
+Calls calls[4];  // [0] FP64, [1] FP32, [2] df64 (double-float), [3] FP32 dual numbers
 }  // namespace wc
 
 #ifdef __CUDA_ARCH__
 #define TCG_COUNT(name)
 #define TCG_COUNT_D(name)
+#define TCG_COUNT_T(name, type)
 #else
 #define TCG_COUNT(name) (::wc::calls[::tcg::Prec<F>::cls].name++)
 #define TCG_COUNT_D(name) (::wc::calls[0].name++)
+#define TCG_COUNT_T(name, type) (::wc::calls[::tcg::Prec<type>::cls].name++)
 #endif
 
 #include "tc_kernels.cuh"
@@ -222,11 +224,11 @@ int main(int argc, char** argv) {
     const wc::Calls& h = wc::calls[2];
     printf("  \"mode%d\": {\"substeps\": %.4f, \"fp64\": {\"chem_T\": %.4f, \"cool_T\": %.4f, \"temp_step\": %.4f, \"equil\": %.4f, "
            "\"equil_it\": %.4f, \"dust\": %.4f, \"dust_it\": %.4f, \"source\": %.4f, \"newton64_it\": %.4f, "
-           "\"chord64_it\": %.4f, \"newton32_it\": %.4f, \"polish_it\": %.4f, \"substep_paper\": %.4f, "
+           "\"chord64_it\": %.4f, \"tangent_it\": %.4f, \"newton32_it\": %.4f, \"polish_it\": %.4f, \"substep_paper\": %.4f, "
            "\"picard_it\": %.4f}, ",
            mode, (double)nsub / n, (double)k.chem_T / n, (double)k.cool_T / n, (double)k.temp_step / n, (double)k.equil / n,
            (double)k.equil_it / n, (double)k.dust / n, (double)k.dust_it / n, (double)k.source / n,
-           (double)k.newton64_it / n, (double)k.chord64_it / n, (double)k.newton32_it / n, (double)k.polish_it / n,
+           (double)k.newton64_it / n, (double)k.chord64_it / n, (double)k.tangent_it / n, (double)k.newton32_it / n, (double)k.polish_it / n,
            (double)k.substep_paper / n, (double)k.picard_it / n);
     for (int cl = 1; cl <= 2; ++cl) {
       const wc::Calls& x = (cl == 1) ? f : h;

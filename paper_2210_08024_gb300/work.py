@@ -12,6 +12,8 @@ scalar type; its counts per iteration are stated here from the code:
     FP64 Newton iteration   63 add, 55 mul, 16 div   (one division per Jacobian column)
     FP64 chord iteration    42 add, 40 mul, 13 div   (the same without the differencing:
                                                       21 add, 15 mul, 9 div)
+    dual-number iteration   11 add,  6 mul           (its FP64 part: residual and step; the
+                                                      Jacobian and the correction are FP32)
     mixed Newton iteration  18 add, 12 mul,  6 div   (its FP64 part: residual, damped step
                                                       and test; the correction is solved in FP32)
     polish iteration        16 add, 12 mul,  6 div   (the same, residual from df64 sources)
@@ -47,6 +49,7 @@ OUT = os.path.join(HERE, "work_slab128.json")
 LINALG = {
     "newton64_it": {"add": 63, "mul": 55, "div": 16},
     "chord64_it": {"add": 42, "mul": 40, "div": 13},
+    "tangent_it": {"add": 11, "mul": 6, "div": 0},
     "newton32_it": {"add": 18, "mul": 12, "div": 6},
     "polish_it": {"add": 16, "mul": 12, "div": 6},
     "substep_paper": {"add": 18, "mul": 18, "div": 8},
@@ -105,7 +108,7 @@ def algorithmic(counts: dict) -> dict:
         k, f, h = counts[mode]["fp64"], counts[mode]["fp32"], counts[mode].get("df64", {})
         ns = counts[mode]["substeps"]
         src = k["source"] + f["source"] + h.get("source", 0.0)
-        its = k["newton64_it"] + k["chord64_it"] + k["newton32_it"]
+        its = k["newton64_it"] + k["chord64_it"] + k["tangent_it"] + k["newton32_it"]
         out[mode] = {"substeps": round(ns, 4), "source_evals": round(src, 3),
                      "source_evals_per_substep": round(src / ns, 3) if ns else 0.0,
                      "fp64_source_evals": round(k["source"], 3),
@@ -157,7 +160,9 @@ def breakdown(res: dict, mode: str = "mode1") -> list:
     for blk, la in LINALG.items():
         n = calls.get(blk, 0.0)
         rows.append((blk, n, n * sum(v * SLOT_WEIGHTS[c] for c, v in la.items())))
-    rows = [r for r in rows if r[2] > 0.0]
+    # the plain iteration's blocks stay listed in mode 1 where the sample never needs it
+    plain = ("temp_step", "newton64_it", "chord64_it") if mode == "mode1" else ()
+    rows = [r for r in rows if r[2] > 0.0 or r[0] in plain]
     return sorted(rows, key=lambda r: -r[2])
 
 
