@@ -1245,12 +1245,14 @@ TCG_FN bool seed_from_outputs(const float* o, const double* g, const LaneState& 
 //   3 blocks (168 registers, compiler's choice) 546 / 403
 //   4 blocks (128) 394 / 195,  5 (96) 375 / 174,  6 (80) 365 / 164,
 //   7 (72) 362 / 156,  8 (64) 363 / 152.
-// The paper scheme is compiled for 6 (80 registers; 4 blocks: 50.7 ms, 5: 50.3, 6: 50.0 when
-// its FP64 exp and log went out of line), the FP64 Newton kernels for 8: with the Jacobian
-// from dual numbers, FP32 work that overlaps the FP64 pipe, 4 / 5 / 6 / 8 blocks took
-// 96.1 / 93.4 / 90.7 / 87.6 ms.  The seeded FP64 kernel keeps 8 (293.5 ms; 300.1 at 6).
+// The paper scheme is compiled for 4 (128 registers): its four large blocks leave the FP64
+// pipe 85% busy at any occupancy, and fewer spills win (a 96^3 slab at 3e3 yr: 3 / 4 / 6
+// blocks 15.6 / 15.5 / 16.9 ms).  The FP64 Newton kernels are compiled for 8: with the
+// Jacobian from dual numbers, FP32 work that overlaps the FP64 pipe, 4 / 5 / 6 / 8 / 10 / 12
+// blocks took 96.1 / 93.4 / 90.7 / 88.2 / 90.8 / 90.9 ms.  The seeded FP64 kernel keeps 8
+// (293.5 ms; 300.1 at 6).
 constexpr int STEP_MIN_BLOCKS = 8;
-constexpr int STEP_MIN_BLOCKS_PAPER = 6;
+constexpr int STEP_MIN_BLOCKS_PAPER = 4;
 // The warp-cooperative kernels (four lanes per cell) serve launches too small to fill
 // the GPU, where the time is the latency of the slowest cells: 4 resident blocks (128
 // registers per thread) spill less.
