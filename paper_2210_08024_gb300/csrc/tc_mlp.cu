@@ -6,10 +6,9 @@
 // BF16, as the step kernel's inference does, and accumulate in FP32.  The weight
 // gradient of the BF16 network is applied to the FP32 masters by Adam.
 //
-// One training step is a handful of small kernels, layer by layer: normalise ->
-// dense+SiLU x3 -> dense -> loss -> back through each layer (input gradient, then
-// weight gradient) -> Adam.  The network is tiny (9155 parameters), so these kernels
-// are plain FP32 FMA loops; the time of the seeded solver is spent in the step kernel.
+// Forward and backward pass are one kernel: a block takes tiles of 64 samples through all
+// layers and back with the weights and the tile's activations in shared memory, and keeps
+// its share of the weight gradients in registers until its last tile.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -77,72 +76,230 @@ __device__ __forceinline__ float silu_d(float z) {
   return s * (1.0f + z * (1.0f - s));
 }
 
-__global__ void k_norm(const float* __restrict__ X, int B, const float* __restrict__ mean,
-                       const float* __restrict__ inv_std, float* __restrict__ A0) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * MLP_IN) return;
-  const int k = i % MLP_IN;
-  A0[i] = (X[i] - mean[k]) * inv_std[k];
-}
+// ------------------------------------------------------------------ the fused pass
+// What bounds it: FP32 FMAs from shared memory (6 x 9411 a sample, 0.46 GFLOP for a batch of
+// 8192: 6 us at the FP32 rate), and for one tile the chain of its seven small products.  As
+// separate kernels per layer (one thread an output, weights read with a 256-byte stride,
+// the weight gradients by a few thousand threads) the same batch took 430 us on the device.
+// Layout: activations are [unit][sample] with rows of TS + 4 floats (16-byte loads; rows
+// read side by side fall into different banks), hidden weights are held in both
+// orientations so that either product reads four neighbouring values at once.  A thread owns
+// 4 units x 4 samples of a layer, or 4 x 4 weights of a gradient: eight 16-byte loads for 64
+// FMAs there.  64 samples: 180 KB of shared memory, and a batch of 8192 is one tile on each of
+// 128 SMs.
+constexpr int TS = 64;          // samples per tile
+constexpr int LD = TS + 4;      // row length of an activation
+constexpr int NT = 256;         // threads per block
+constexpr int HID = MLP_HID;
+static_assert(HID == 64 && MLP_OUT == 3 && MLP_IN <= 16, "thread maps below");
 
-// Z[b][n] = b[n] + sum_k bf16(W[n][k]) A[b][k]; H = silu(Z) when act.
-__global__ void k_fwd(const float* __restrict__ A, int K, const float* __restrict__ W, const float* __restrict__ bias,
-                      int N, int B, float* __restrict__ Z, float* __restrict__ H, bool act) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * N) return;
-  const int b = i / N, n = i % N;
-  float acc = bias[n];
-  for (int k = 0; k < K; ++k) acc = fmaf(bf(W[n * K + k]), A[b * K + k], acc);
-  Z[i] = acc;
-  if (act) H[i] = tcg::mlp_silu(acc);
-}
+struct Smem {
+  float W1t[MLP_IN * LD], W2t[HID * LD], W3t[HID * LD];  // [in][out], rows of LD
+  float W2[HID * HID], W3[HID * HID];                    // [out][in]
+  float W4[MLP_OUT * HID];
+  float b1[HID], b2[HID], b3[HID], b4[4];
+  float A0[MLP_IN * LD];
+  float H1[HID * LD], H2[HID * LD], H3[HID * LD];
+  float Z1[HID * LD], Z2[HID * LD], Z3[HID * LD];  // pre-activations, then the gradients to them
+  float G[MLP_OUT * LD];
+};
 
-// G[b][m] = 2 w_m (O - Y) / B; loss += sum w_m (O - Y)^2 / B.
-__global__ void k_loss(const float* __restrict__ O, const float* __restrict__ Y, int B, float w0, float w1, float w2,
-                       float* __restrict__ G, float* __restrict__ loss) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float l = 0.f;
-  if (i < B * MLP_OUT) {
-    const int m = i % MLP_OUT;
-    const float w = (m == 0) ? w0 : (m == 1) ? w1 : w2;
-    const float d = O[i] - Y[i];
-    G[i] = 2.f * w * d / (float)B;
-    l = w * d * d / (float)B;
+// Z[n][s] = b[n] + sum_k Wt[k][n] A[k][s] in the order of k; H = silu(Z).
+template <int K>
+__device__ __forceinline__ void layer_fwd(const float* __restrict__ A, const float* __restrict__ Wt,
+                                          const float* __restrict__ bias, float* __restrict__ Z,
+                                          float* __restrict__ H) {
+  const int s0 = 4 * (threadIdx.x & 15), n0 = 4 * (threadIdx.x >> 4);
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = bias[n0 + i];
+#pragma unroll 8
+  for (int k = 0; k < K; ++k) {
+    const float4 a = *reinterpret_cast<const float4*>(A + k * LD + s0);
+    const float4 w = *reinterpret_cast<const float4*>(Wt + k * LD + n0);
+    const float av[4] = {a.x, a.y, a.z, a.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(wv[i], av[j], acc[i][j]);
   }
-  for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
-  if ((threadIdx.x & 31) == 0 && l != 0.f) atomicAdd(loss, l);
-}
-
-// Gin[b][k] = (sum_n Gout[b][n] bf16(W[n][k])) * silu'(Zin[b][k])
-__global__ void k_bwd_data(const float* __restrict__ Gout, int N, const float* __restrict__ W, int K,
-                           const float* __restrict__ Zin, int B, float* __restrict__ Gin) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= B * K) return;
-  const int b = i / K, k = i % K;
-  float acc = 0.f;
-  for (int n = 0; n < N; ++n) acc = fmaf(Gout[b * N + n], bf(W[n * K + k]), acc);
-  Gin[i] = acc * silu_d(Zin[i]);
-}
-
-// dW[n][k] = sum_b Gout[b][n] A[b][k]; db[n] = sum_b Gout[b][n].  One thread per (n, k)
-// (plus one per n for the bias), each summing over a slice of the batch; slices are
-// combined with atomicAdd.
-__global__ void k_bwd_w(const float* __restrict__ Gout, int N, const float* __restrict__ A, int K, int B, int bslice,
-                        float* __restrict__ dW, float* __restrict__ db) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int b0 = blockIdx.y * bslice;
-  const int b1 = min(B, b0 + bslice);
-  if (i < N * K) {
-    const int n = i / K, k = i % K;
-    float acc = 0.f;
-    for (int b = b0; b < b1; ++b) acc = fmaf(Gout[b * N + n], A[b * K + k], acc);
-    atomicAdd(&dW[i], acc);
-  } else if (i < N * K + N) {
-    const int n = i - N * K;
-    float acc = 0.f;
-    for (int b = b0; b < b1; ++b) acc += Gout[b * N + n];
-    atomicAdd(&db[n], acc);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float4 z = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]};
+    float4 h = {tcg::mlp_silu(z.x), tcg::mlp_silu(z.y), tcg::mlp_silu(z.z), tcg::mlp_silu(z.w)};
+    *reinterpret_cast<float4*>(Z + (n0 + i) * LD + s0) = z;
+    *reinterpret_cast<float4*>(H + (n0 + i) * LD + s0) = h;
   }
+}
+
+// Z[k][s] <- (sum_n G[n][s] W[n][k]) silu'(Z[k][s]): each thread replaces its own values.
+template <int N>
+__device__ __forceinline__ void layer_bwd(const float* __restrict__ G, const float* __restrict__ W,
+                                          float* __restrict__ Z) {
+  const int s0 = 4 * (threadIdx.x & 15), k0 = 4 * (threadIdx.x >> 4);
+  float acc[4][4] = {};
+#pragma unroll 8
+  for (int n = 0; n < N; ++n) {
+    const float4 g = *reinterpret_cast<const float4*>(G + n * LD + s0);
+    const float4 w = *reinterpret_cast<const float4*>(W + n * HID + k0);
+    const float gv[4] = {g.x, g.y, g.z, g.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(gv[j], wv[i], acc[i][j]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float4* zp = reinterpret_cast<float4*>(Z + (k0 + i) * LD + s0);
+    const float4 z = *zp;
+    *zp = float4{acc[i][0] * silu_d(z.x), acc[i][1] * silu_d(z.y), acc[i][2] * silu_d(z.z), acc[i][3] * silu_d(z.w)};
+  }
+}
+
+__device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+
+// dW[n][k] += sum_s G[n][s] A[k][s] for n = 4 (t / 16) + i, k = t % 16 + 16 j; db[n] += sum_s G[n][s].
+__device__ __forceinline__ void layer_dw(const float* __restrict__ G, const float* __restrict__ A, float (&dw)[4][4],
+                                         float (&db)[4]) {
+  const int kx = threadIdx.x & 15, n0 = 4 * (threadIdx.x >> 4);
+#pragma unroll 4
+  for (int s = 0; s < TS; s += 4) {
+    float4 g[4], a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g[i] = *reinterpret_cast<const float4*>(G + (n0 + i) * LD + s);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] = *reinterpret_cast<const float4*>(A + (kx + 16 * j) * LD + s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      db[i] += (g[i].x + g[i].y) + (g[i].z + g[i].w);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) dw[i][j] = dot4(g[i], a[j], dw[i][j]);
+    }
+  }
+}
+
+// The forward pass of B rows of X (out, when given, receives the outputs), and with TRAIN
+// the loss sum_b sum_m w_m (O - Y)^2 / B and its gradient, both added to what grad and loss
+// hold.
+template <bool TRAIN>
+__global__ void __launch_bounds__(NT) k_pass(const float* __restrict__ theta, const float* __restrict__ norm,
+                                             const float* __restrict__ X, const float* __restrict__ Y, int B, float w0,
+                                             float w1, float w2, float* __restrict__ out, float* __restrict__ grad,
+                                             float* __restrict__ loss) {
+  extern __shared__ float4 smem_raw[];
+  Smem& m = *reinterpret_cast<Smem*>(smem_raw);
+  const int t = threadIdx.x;
+  for (int i = t; i < HID * MLP_IN; i += NT) m.W1t[(i % MLP_IN) * LD + i / MLP_IN] = bf(theta[OFF_W1 + i]);
+  for (int i = t; i < HID * HID; i += NT) {
+    const int o = i / HID, k = i % HID;
+    const float v2 = bf(theta[OFF_W2 + i]), v3 = bf(theta[OFF_W3 + i]);
+    m.W2t[k * LD + o] = v2;
+    m.W3t[k * LD + o] = v3;
+    if (TRAIN) {
+      m.W2[i] = v2;
+      m.W3[i] = v3;
+    }
+  }
+  for (int i = t; i < MLP_OUT * HID; i += NT) m.W4[i] = bf(theta[OFF_W4 + i]);
+  if (t < HID) {
+    m.b1[t] = theta[OFF_B1 + t];
+    m.b2[t] = theta[OFF_B2 + t];
+    m.b3[t] = theta[OFF_B3 + t];
+  }
+  if (t < MLP_OUT) m.b4[t] = theta[OFF_B4 + t];
+  float dw1[4] = {}, db1 = 0.f, dw2[4][4] = {}, db2[4] = {}, dw3[4][4] = {}, db3[4] = {}, dw4 = 0.f, db4 = 0.f;
+  float lsum = 0.f;
+  for (long long b0 = (long long)blockIdx.x * TS; b0 < B; b0 += (long long)gridDim.x * TS) {
+    const int live = (B - b0 < TS) ? int(B - b0) : TS;
+    __syncthreads();  // the last tile's gradients are done with the activations
+    for (int i = t; i < TS * MLP_IN; i += NT) {
+      const int s = i / MLP_IN, k = i % MLP_IN;
+      m.A0[k * LD + s] = (s < live) ? (X[b0 * MLP_IN + i] - norm[k]) * norm[MLP_IN + k] : 0.f;
+    }
+    __syncthreads();
+    layer_fwd<MLP_IN>(m.A0, m.W1t, m.b1, m.Z1, m.H1);
+    __syncthreads();
+    layer_fwd<HID>(m.H1, m.W2t, m.b2, m.Z2, m.H2);
+    __syncthreads();
+    layer_fwd<HID>(m.H2, m.W3t, m.b3, m.Z3, m.H3);
+    __syncthreads();
+    if (t < MLP_OUT * TS) {  // the output layer: one output of one sample a thread
+      const int o = t / TS, s = t % TS;
+      float acc = m.b4[o];
+#pragma unroll 8
+      for (int k = 0; k < HID; ++k) acc = fmaf(m.W4[o * HID + k], m.H3[k * LD + s], acc);
+      const long long r = (b0 + s) * MLP_OUT + o;
+      if (out && s < live) out[r] = acc;
+      if (TRAIN) {
+        const float w = (o == 0) ? w0 : (o == 1) ? w1 : w2;
+        const float d = (s < live) ? acc - Y[r] : 0.f;
+        m.G[o * LD + s] = 2.f * w * d / (float)B;
+        lsum += w * d * d / (float)B;
+      }
+    }
+    if (!TRAIN) continue;
+    __syncthreads();
+    if (t < MLP_OUT * HID) {
+      const int o = t / HID, k = t % HID;
+#pragma unroll 4
+      for (int s = 0; s < TS; s += 4) {
+        const float4 g = *reinterpret_cast<const float4*>(m.G + o * LD + s);
+        dw4 = dot4(g, *reinterpret_cast<const float4*>(m.H3 + k * LD + s), dw4);
+        db4 += (g.x + g.y) + (g.z + g.w);
+      }
+    }
+    layer_bwd<MLP_OUT>(m.G, m.W4, m.Z3);
+    __syncthreads();
+    layer_dw(m.Z3, m.H2, dw3, db3);
+    layer_bwd<HID>(m.Z3, m.W3, m.Z2);
+    __syncthreads();
+    layer_dw(m.Z2, m.H1, dw2, db2);
+    layer_bwd<HID>(m.Z2, m.W2, m.Z1);
+    __syncthreads();
+    {  // first layer: unit t / 4, inputs t % 4 + 4 j
+      const int n = t >> 2, k0 = t & 3;
+#pragma unroll 4
+      for (int s = 0; s < TS; s += 4) {
+        const float4 g = *reinterpret_cast<const float4*>(m.Z1 + n * LD + s);
+        db1 += (g.x + g.y) + (g.z + g.w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (k0 + 4 * j < MLP_IN)
+            dw1[j] = dot4(g, *reinterpret_cast<const float4*>(m.A0 + (k0 + 4 * j) * LD + s), dw1[j]);
+      }
+    }
+  }
+  if (!TRAIN) return;
+  {
+    const int kx = t & 15, n0 = 4 * (t >> 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        atomicAdd(grad + OFF_W2 + (n0 + i) * HID + kx + 16 * j, dw2[i][j]);
+        atomicAdd(grad + OFF_W3 + (n0 + i) * HID + kx + 16 * j, dw3[i][j]);
+      }
+      if (kx == 0) {
+        atomicAdd(grad + OFF_B2 + n0 + i, db2[i]);
+        atomicAdd(grad + OFF_B3 + n0 + i, db3[i]);
+      }
+    }
+    if (t < MLP_OUT * HID) {
+      atomicAdd(grad + OFF_W4 + t, dw4);
+      if (t % HID == 0) atomicAdd(grad + OFF_B4 + t / HID, db4);
+    }
+    const int n = t >> 2, k0 = t & 3;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (k0 + 4 * j < MLP_IN) atomicAdd(grad + OFF_W1 + n * MLP_IN + k0 + 4 * j, dw1[j]);
+    if (k0 == 0) atomicAdd(grad + OFF_B1 + n, db1);
+  }
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+  if ((t & 31) == 0 && lsum != 0.f) atomicAdd(loss, lsum);
 }
 
 __global__ void k_adam(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
@@ -168,87 +325,16 @@ struct tc_mlp {
   float* v = nullptr;
   float* norm = nullptr;   // mean[MLP_IN], inv_std[MLP_IN]
   float* loss = nullptr;
-  float* work = nullptr;   // activations for cap samples
-  int cap = 0;
+  int num_sms = 1;
   long long t = 0;         // Adam step count
   float h_mean[MLP_IN], h_inv_std[MLP_IN];
 };
 
 namespace {
 
-// Work layout for B samples: A0[B*MLP_IN] Z1 H1 Z2 H2 Z3 H3 [B*64 each] O G[B*3] G3 G2 G1 [B*64].
-size_t work_floats(int B) { return (size_t)B * (MLP_IN + 6 * MLP_HID + 2 * MLP_OUT + 3 * MLP_HID); }
-
-int ensure_cap(tc_mlp* h, int B) {
-  if (B <= h->cap) return TC_OK;
-  cudaFree(h->work);
-  h->work = nullptr;
-  h->cap = 0;
-  if (cudaMalloc(&h->work, work_floats(B) * sizeof(float)) != cudaSuccess) return TC_ENOMEM;
-  h->cap = B;
-  return TC_OK;
-}
-
-struct Bufs {
-  float *A0, *Z1, *H1, *Z2, *H2, *Z3, *H3, *O, *G, *G3, *G2, *G1;
-};
-
-Bufs bufs(tc_mlp* h, int B) {
-  Bufs b;
-  float* p = h->work;
-  b.A0 = p; p += (size_t)B * MLP_IN;
-  b.Z1 = p; p += (size_t)B * MLP_HID;
-  b.H1 = p; p += (size_t)B * MLP_HID;
-  b.Z2 = p; p += (size_t)B * MLP_HID;
-  b.H2 = p; p += (size_t)B * MLP_HID;
-  b.Z3 = p; p += (size_t)B * MLP_HID;
-  b.H3 = p; p += (size_t)B * MLP_HID;
-  b.O = p; p += (size_t)B * MLP_OUT;
-  b.G = p; p += (size_t)B * MLP_OUT;
-  b.G3 = p; p += (size_t)B * MLP_HID;
-  b.G2 = p; p += (size_t)B * MLP_HID;
-  b.G1 = p;
-  return b;
-}
-
-int forward(tc_mlp* h, const float* X, int B, cudaStream_t st, Bufs& b) {
-  const int T = 256;
-  k_norm<<<blocks((long long)B * MLP_IN, T), T, 0, st>>>(X, B, h->norm, h->norm + MLP_IN, b.A0);
-  k_fwd<<<blocks((long long)B * MLP_HID, T), T, 0, st>>>(b.A0, MLP_IN, h->theta + OFF_W1, h->theta + OFF_B1, MLP_HID,
-                                                          B, b.Z1, b.H1, true);
-  k_fwd<<<blocks((long long)B * MLP_HID, T), T, 0, st>>>(b.H1, MLP_HID, h->theta + OFF_W2, h->theta + OFF_B2, MLP_HID,
-                                                          B, b.Z2, b.H2, true);
-  k_fwd<<<blocks((long long)B * MLP_HID, T), T, 0, st>>>(b.H2, MLP_HID, h->theta + OFF_W3, h->theta + OFF_B3, MLP_HID,
-                                                          B, b.Z3, b.H3, true);
-  k_fwd<<<blocks((long long)B * MLP_OUT, T), T, 0, st>>>(b.H3, MLP_HID, h->theta + OFF_W4, h->theta + OFF_B4, MLP_OUT,
-                                                          B, b.O, nullptr, false);
-  return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
-}
-
-int backward(tc_mlp* h, const float* Y, int B, const float* w3, cudaStream_t st, Bufs& b) {
-  const int T = 256;
-  if (cudaMemsetAsync(h->grad, 0, NPARAM * sizeof(float), st) != cudaSuccess) return TC_ECUDA;
-  if (cudaMemsetAsync(h->loss, 0, sizeof(float), st) != cudaSuccess) return TC_ECUDA;
-  const float w0 = w3 ? w3[0] : 1.f, w1 = w3 ? w3[1] : 1.f, w2 = w3 ? w3[2] : 1.f;
-  k_loss<<<blocks((long long)B * MLP_OUT, T), T, 0, st>>>(b.O, Y, B, w0, w1, w2, b.G, h->loss);
-  const int bs = 512;
-  const int ns = (B + bs - 1) / bs;
-  // output layer
-  k_bwd_w<<<dim3(blocks(MLP_OUT * MLP_HID + MLP_OUT, T), ns), T, 0, st>>>(b.G, MLP_OUT, b.H3, MLP_HID, B, bs,
-                                                                            h->grad + OFF_W4, h->grad + OFF_B4);
-  k_bwd_data<<<blocks((long long)B * MLP_HID, T), T, 0, st>>>(b.G, MLP_OUT, h->theta + OFF_W4, MLP_HID, b.Z3, B, b.G3);
-  // hidden layer 3
-  k_bwd_w<<<dim3(blocks(MLP_HID * MLP_HID + MLP_HID, T), ns), T, 0, st>>>(b.G3, MLP_HID, b.H2, MLP_HID, B, bs,
-                                                                            h->grad + OFF_W3, h->grad + OFF_B3);
-  k_bwd_data<<<blocks((long long)B * MLP_HID, T), T, 0, st>>>(b.G3, MLP_HID, h->theta + OFF_W3, MLP_HID, b.Z2, B, b.G2);
-  // hidden layer 2
-  k_bwd_w<<<dim3(blocks(MLP_HID * MLP_HID + MLP_HID, T), ns), T, 0, st>>>(b.G2, MLP_HID, b.H1, MLP_HID, B, bs,
-                                                                            h->grad + OFF_W2, h->grad + OFF_B2);
-  k_bwd_data<<<blocks((long long)B * MLP_HID, T), T, 0, st>>>(b.G2, MLP_HID, h->theta + OFF_W2, MLP_HID, b.Z1, B, b.G1);
-  // hidden layer 1
-  k_bwd_w<<<dim3(blocks(MLP_HID * MLP_IN + MLP_HID, T), ns), T, 0, st>>>(b.G1, MLP_HID, b.A0, MLP_IN, B, bs,
-                                                                           h->grad + OFF_W1, h->grad + OFF_B1);
-  return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
+int pass_grid(const tc_mlp* h, int B) {
+  const long long tiles = ((long long)B + TS - 1) / TS;
+  return (int)(tiles < h->num_sms ? tiles : h->num_sms);
 }
 
 // splitmix64 (Steele, Lea & Flood 2014) for a reproducible weight initialisation.
@@ -275,6 +361,13 @@ int tc_mlp_create(unsigned long long seed, tc_mlp** out) {
             cudaMalloc(&h->v, NPARAM * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&h->norm, 2 * MLP_IN * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&h->loss, sizeof(float)) == cudaSuccess;
+  int dev = 0;
+  ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
+       cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+       cudaFuncSetAttribute(k_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)) ==
+           cudaSuccess &&
+       cudaFuncSetAttribute(k_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem)) ==
+           cudaSuccess;
   if (!ok) {
     tc_mlp_destroy(h);
     return TC_ENOMEM;
@@ -317,7 +410,6 @@ void tc_mlp_destroy(tc_mlp* h) {
   cudaFree(h->v);
   cudaFree(h->norm);
   cudaFree(h->loss);
-  cudaFree(h->work);
   delete h;
 }
 
@@ -349,31 +441,22 @@ int tc_mlp_get_params(const tc_mlp* h, float* theta) {
 int tc_mlp_predict(tc_mlp* h, const float* X, int B, float* out, void* stream) {
   if (!h || B < 0 || (B > 0 && (!X || !out))) return TC_EINVAL;
   if (B == 0) return TC_OK;
-  int rc = ensure_cap(h, B);
-  if (rc != TC_OK) return rc;
-  cudaStream_t st = (cudaStream_t)stream;
-  Bufs b = bufs(h, B);
-  rc = forward(h, X, B, st, b);
-  if (rc != TC_OK) return rc;
-  return cudaMemcpyAsync(out, b.O, (size_t)B * MLP_OUT * sizeof(float), cudaMemcpyDeviceToDevice, st) == cudaSuccess
-             ? TC_OK : TC_ECUDA;
+  k_pass<false><<<pass_grid(h, B), NT, sizeof(Smem), (cudaStream_t)stream>>>(h->theta, h->norm, X, nullptr, B, 0.f, 0.f,
+                                                                             0.f, out, nullptr, nullptr);
+  return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
 }
 
 int tc_mlp_grad(tc_mlp* h, const float* X, const float* Y, int B, const float* w3, float* grad, float* loss,
                 void* stream) {
   if (!h || B < 1 || !X || !Y) return TC_EINVAL;
-  int rc = ensure_cap(h, B);
-  if (rc != TC_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  Bufs b = bufs(h, B);
-  rc = forward(h, X, B, st, b);
-  if (rc == TC_OK) rc = backward(h, Y, B, w3, st, b);
-  if (rc != TC_OK) return rc;
-  if (grad && cudaMemcpyAsync(grad, h->grad, NPARAM * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return TC_ECUDA;
-  if (loss && cudaMemcpyAsync(loss, h->loss, sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-    return TC_ECUDA;
-  return TC_OK;
+  float* g = grad ? grad : h->grad;
+  float* l = loss ? loss : h->loss;
+  if (cudaMemsetAsync(g, 0, NPARAM * sizeof(float), st) != cudaSuccess) return TC_ECUDA;
+  if (cudaMemsetAsync(l, 0, sizeof(float), st) != cudaSuccess) return TC_ECUDA;
+  const float w0 = w3 ? w3[0] : 1.f, w1 = w3 ? w3[1] : 1.f, w2 = w3 ? w3[2] : 1.f;
+  k_pass<true><<<pass_grid(h, B), NT, sizeof(Smem), st>>>(h->theta, h->norm, X, Y, B, w0, w1, w2, nullptr, g, l);
+  return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
 }
 
 int tc_mlp_train_step(tc_mlp* h, const float* X, const float* Y, int B, const float* w3, float lr, float* loss,
