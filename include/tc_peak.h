@@ -7,7 +7,7 @@
  * independent dependency chains of `iters` operations.  The caller times it (CUDA
  * events on the same stream).  Operations per launch = grid * block * chains * iters.
  *   kind 0: FP64 fused multiply-add      kind 1: FP32 fused multiply-add
- *   kind 2: FP64 exp()                   kind 3: FP64 log()
+ *   kind 2: FP64 exp (the step's, tc_exp64.cuh)  kind 3: FP64 log (the same)
  *   kind 4: FP64 sqrt()                  kind 5: FP64 division
  *   kind 6: FP64 pow(x, y)               kind 7: FP32 expf()
  *   kind 8: FP32 __expf(), the approximate exponential of the fast-math mixed kernels:

@@ -1,5 +1,9 @@
 // Instantiation of the warp-cooperative mode-2 step kernel (four lanes per cell; see
 // tc_kernels.cuh).  Built with fast FP32 intrinsics like the other mixed kernels.
+// FP64 runs only in this kernel's rare fallbacks: exp() and log() keep its code, bound by
+// instruction fetch, as it was (with the tables of tc_exp64.cuh the seeded mixed step on the
+// 128^3 slab took 55.5 ms against 51.5).
+#define TCG_PLAIN_EXP64
 #include "tc_launch.h"
 
 namespace tcg {

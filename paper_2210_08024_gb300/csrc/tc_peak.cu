@@ -5,6 +5,7 @@
 
 #include "../../include/tc.h"
 #include "../../include/tc_peak.h"
+#include "tc_exp64.cuh"
 
 namespace tcg {
 int df64_peak_launch(int kind, int grid, int block, int iters, double* sink, void* stream);  // tc_df64_diag.cu
@@ -38,8 +39,8 @@ __global__ void k_peak(int iters, double* sink) {
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
         if (KIND == 0) v[c] = fma(v[c], a, b);
-        if (KIND == 2) v[c] = exp(-v[c]);          // converges to the omega constant
-        if (KIND == 3) v[c] = log(v[c] + 2.0);      // converges to ~1.146
+        if (KIND == 2) v[c] = tcg::exp64(-v[c]);          // converges to the omega constant
+        if (KIND == 3) v[c] = tcg::log64(v[c] + 2.0);      // converges to ~1.146
         if (KIND == 4) v[c] = sqrt(v[c] + 1.0);     // converges to the golden ratio
         if (KIND == 5) v[c] = 1.0 / (v[c] + 1.0);   // converges to 0.618
         if (KIND == 6) v[c] = pow(v[c] + 1.0, 0.7);

@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include "tc_df64.cuh"
+#include "tc_exp64.cuh"
 
 // Physics and substep functions are host+device so the host compiler can also build
 // them (used by the host-side test harness of the library's own kernels).
@@ -63,11 +64,17 @@ constexpr double FOURPI = 12.566370614359172;
 constexpr unsigned FL_CONST_KGR = 1u, FL_NO_ROVIB = 2u, FL_NO_CIE = 4u;
 
 // ------------------------------------------------------------------ precision-generic math
-// FP64 exp and log are called out of line on the device: the physics blocks hold ~50
-// call sites, and one shared copy keeps the kernels' code smaller (instruction fetch;
-// FP64 Newton step on the 128^3 slab 232.5 -> 226.5 ms).
-__device__ __noinline__ inline double m_exp64_ool(double x) { return exp(x); }
-__device__ __noinline__ inline double m_log64_ool(double x) { return log(x); }
+// FP64 exp and log are the table-driven ones of tc_exp64.cuh on the device, called out of
+// line: the physics blocks hold ~50 call sites, and one shared copy keeps the kernels' code
+// smaller (instruction fetch; with exp() and log() out of line the FP64 Newton step on the
+// 128^3 slab took 226.5 ms, inlined 232.5).
+#ifdef TCG_PLAIN_EXP64
+__device__ __noinline__ static double m_exp64_ool(double x) { return exp(x); }
+__device__ __noinline__ static double m_log64_ool(double x) { return log(x); }
+#else
+__device__ __noinline__ static double m_exp64_ool(double x) { return exp64(x); }
+__device__ __noinline__ static double m_log64_ool(double x) { return log64(x); }
+#endif
 TCG_FN double m_exp(double x) {
 #ifdef __CUDA_ARCH__
   return m_exp64_ool(x);
