@@ -9,7 +9,8 @@
 // The Jacobian only steers the iteration; residuals, updates and roots stay in FP64.
 //
 // On the device the elementary functions are the approximate FP32 ones (errors of a few
-// 1e-7, growing as 1e-7 |x| in the exponential).  Comparisons look at the value alone.
+// 1e-7, growing as 1e-7 |x| in the exponential).  Literal constants and the cell's
+// constants stay plain FP32 values.  Comparisons look at the value alone.
 #pragma once
 #include "tc_phys.cuh"
 
@@ -32,25 +33,45 @@ template <> struct Prec<dualf> {
   static constexpr int cls = 3;
 };
 
+template <> struct ConstOf<dualf> { using type = float; };
+
+// One MUFU instruction each on the device (with a scaling multiply for exp and log), by PTX:
+// the intrinsics of a build without fast math wrap them in range handling.  Subnormal
+// arguments and results flush to zero.
 TCG_FN float dual_rcp(float x) {
 #ifdef __CUDA_ARCH__
-  return __fdividef(1.0f, x);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 #else
   return 1.0f / x;
 #endif
 }
 TCG_FN float dual_exp(float x) {
 #ifdef __CUDA_ARCH__
-  return __expf(x);
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.44269504f));
+  return r;
 #else
   return expf(x);
 #endif
 }
 TCG_FN float dual_log(float x) {
 #ifdef __CUDA_ARCH__
-  return __logf(x);
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r * 0.693147181f;
 #else
   return logf(x);
+#endif
+}
+TCG_FN float dual_sqrt(float x) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+#else
+  return sqrtf(x);
 #endif
 }
 
@@ -89,11 +110,13 @@ TCG_FN dualf m_exp(dualf x) {
 }
 TCG_FN dualf m_log(dualf x) { return dualf::make(dual_log(x.v), x.d * dual_rcp(x.v)); }
 TCG_FN dualf m_sqrt(dualf x) {
-  const float s = sqrtf(x.v);
+  const float s = dual_sqrt(x.v);
   return dualf::make(s, 0.5f * x.d * dual_rcp(s));
 }
 TCG_FN dualf m_max(dualf a, dualf b) { return (a.v < b.v) ? b : a; }
 TCG_FN dualf m_min(dualf a, dualf b) { return (b.v < a.v) ? b : a; }
+TCG_FN dualf m_max(dualf a, float b) { return (a.v < b) ? dualf::make(b, 0.0f) : a; }
+TCG_FN dualf m_min(dualf a, float b) { return (b < a.v) ? dualf::make(b, 0.0f) : a; }
 TCG_FN dualf m_abs(dualf a) { return (a.v < 0.0f) ? -a : a; }
 
 // The C/O/e equilibrium along one direction, given its root x_e.  With g(x; y) the
@@ -146,16 +169,18 @@ TCG_FN dualf dust_tangent(const CellC<float>& c, const ChemT<dualf>& b, float td
 
 // Derivatives of f = (H/K, C_H2, C_H+) and of (x_e, x_C+, x_CO) along ln T, x_H2 and x_H+
 // at one state, given its x_e and dust temperature: df[i][j] and dq[i][j], j the
-// direction.  The temperature blocks are differentiated once; the two abundance
-// directions run on them with their derivatives cleared.  `hk` is 1 / (mu_H k_B / (gamma
-// - 1)): H/K = (Gamma - n Lambda) hk stays in FP32's range at any density.
+// direction, for the directions j0 <= j < j1.  The temperature blocks are differentiated
+// once; the two abundance directions run on them with their derivatives cleared.  `hk` is
+// 1 / (mu_H k_B / (gamma - 1)): H/K = (Gamma - n Lambda) hk stays in FP32's range at any
+// density.
 TCG_BIG inline void source_tangents(const CellC<float>& c, unsigned flags, float hk, float T, float x2, float xp,
-                                    float xH, float xe, float td, float (*df)[3], float (*dq)[3]) {
-  ChemT<dualf> b = chem_T(c, dualf::make(T, T), flags);
+                                    float xH, float xe, float td, float (*df)[3], float (*dq)[3], int j0 = 0,
+                                    int j1 = 3) {
+  ChemT<dualf> b = chem_T(c, dualf::make(T, (j0 == 0) ? T : 0.0f), flags);
   CoolT<dualf> k = cool_T(c, b, flags);
 #pragma unroll 1
-  for (int j = 0; j < 3; ++j) {
-    if (j == 1) {
+  for (int j = j0; j < j1; ++j) {
+    if (j == 1 && j0 == 0) {
       dualf* pb = reinterpret_cast<dualf*>(&b);
       dualf* pk = reinterpret_cast<dualf*>(&k);
       for (int i = 0; i < int(sizeof(b) / sizeof(dualf)); ++i) pb[i].d = 0.0f;

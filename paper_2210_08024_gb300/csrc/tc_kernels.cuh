@@ -551,6 +551,7 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 // iteration halves, which changed the substep grid of 5 in 13,824 cells near x_H = 0.)
 constexpr int TAN_MAXIT = 12;
 constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
+template <int LPC = 1>
 TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double mu, double Kinv,
                           const double* yn, double dts, const double* src, double* y, double& xe_g, double& td_g,
                           Equil<double>* qb) {
@@ -568,7 +569,24 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
     const double xH = 1.0 - 2.0 * y[1] - y[2];
     const float y0 = float(y[0]), x2 = float(y[1]), xp = float(y[2]);
     float df[3][3], dq[3][3];
-    source_tangents(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), df, dq);
+    if constexpr (LPC == 4) {
+      // the cell's lanes take one direction each (the last repeats the third) and exchange
+      const int q = lane_in_cell<4>(), j = (q < 3) ? q : 2;
+      float tf[3][3], tq[3][3];
+      source_tangents(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), tf, tq, j, j + 1);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float vf = (j == 0) ? tf[i][0] : (j == 1) ? tf[i][1] : tf[i][2];
+        const float vq = (j == 0) ? tq[i][0] : (j == 1) ? tq[i][1] : tq[i][2];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          df[i][r] = from_lane<4>(vf, r);
+          dq[i][r] = from_lane<4>(vq, r);
+        }
+      }
+    } else {
+      source_tangents(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), df, dq);
+    }
     // rows scaled: (T_mu equation / T_mu, x_H2, x_H+); unknowns (ln T_mu, x_H2, x_H+)
     const float iy0 = 1.0f / y0, h = float(dts);
     float J[3][3], r[3], u[3];
@@ -890,7 +908,7 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
   }
   if (src) {
     double xg = xe_g, tg = td_g;
-    it = newton_tangent(c, *cf, p, s.mu, Kinv, yn, dts, src, y, xg, tg, &qb);
+    it = newton_tangent<LPC>(c, *cf, p, s.mu, Kinv, yn, dts, src, y, xg, tg, &qb);
     if (it >= 0) { xe_g = xg; td_g = tg; }
   }
   if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);

@@ -121,6 +121,10 @@ template <> struct Prec<df64> {
   static constexpr int cls = 2;
 };
 
+// Type of the literal constants in code on F (dual numbers take theirs as FP32 values,
+// which have no derivative to carry).
+template <class F> struct ConstOf { using type = F; };
+
 // A value computed at run time, in precision F (df64 keeps subnormal trailing parts on
 // the device; constants convert at compile time with F(x)).
 template <class F> TCG_FN F to_prec(double x) { return F(x); }
@@ -261,42 +265,44 @@ template <class F> struct ChemT {
 // 4.95, whose exponentials differ by the constant factor exp(0.5/0.06)) + Z'_g
 // x_e,metal,CIE (one step at 5.5).
 template <class F, class FC> TCG_FN F xe_hot_of(const CellC<FC>& c, F lt) {
-  F eHe = m_exp((F(4.45) - lt) * F(1.0 / 0.06));
-  F xeHe = F(0.1) * (F(1) / (F(1) + eHe) + F(1) / (F(1) + eHe * F(4160.262005375057)));  // exp(25/3)
-  F xeMet = F(0.012) * logistic((lt - F(5.5)) * F(4));
+  using K = typename ConstOf<F>::type;
+  F eHe = m_exp((K(4.45) - lt) * K(1.0 / 0.06));
+  F xeHe = K(0.1) * (K(1) / (K(1) + eHe) + K(1) / (K(1) + eHe * K(4160.262005375057)));  // exp(25/3)
+  F xeMet = K(0.012) * logistic((lt - K(5.5)) * K(4));
   return xeHe + c.Zg * xeMet;
 }
 
 template <class F, class FC> TCG_BIG ChemT<F> chem_T(const CellC<FC>& c, F T, unsigned flags) {
   TCG_COUNT(chem_T);
+  using K = typename ConstOf<F>::type;
   ChemT<F> b;
   b.T = T;
   b.lnT = m_log(T);
   b.sqT = m_sqrt(T);
-  const F invT = F(1) / T;
+  const F invT = K(1) / T;
   b.invT = invT;
-  b.S = F(1) / (F(1) + m_exp(F(-10.0 / 1.5e4) * (T - F(2.75e4))));
+  b.S = K(1) / (K(1) + m_exp(K(-10.0 / 1.5e4) * (T - K(2.75e4))));
   if (flags & FL_CONST_KGR) {
-    b.kgr = F(3.0e-17) * c.Zd;
+    b.kgr = K(3.0e-17) * c.Zd;
   } else {
-    F s2 = b.sqT * F(0.1);  // sqrt(T/100)
-    F T2 = T * F(0.01);
-    b.kgr = F(3.0e-17) * c.Zd * F(2) * s2 / (F(1) + F(0.4) * s2 + F(0.2) * T2 + F(0.08) * T2 * T2);
+    F s2 = b.sqT * K(0.1);  // sqrt(T/100)
+    F T2 = T * K(0.01);
+    b.kgr = K(3.0e-17) * c.Zd * K(2) * s2 / (K(1) + K(0.4) * s2 + K(0.2) * T2 + K(0.08) * T2 * T2);
   }
-  F lT4 = b.lnT - F(9.210340371976184);  // ln(T/1e4)
-  b.arr = F(2.54e-13) * m_exp((F(-0.8163) - F(0.0208) * lT4) * lT4);
-  b.kci = F(5.85e-11) * b.sqT * m_exp(F(-157809.1) * invT) / (F(1) + b.sqT * F(0.003162277660168379));
-  b.kcdH = F(6.67e-12) * b.sqT * m_exp(F(-1) - F(63593.0) * invT);
-  b.kcdH2 = F(5.996e-30) * m_exp(F(4.1881) * b.lnT - F(54657.4) * invT - F(5.6881) * m_log(F(1) + F(6.761e-6) * T));
-  F lT300 = b.lnT - F(5.703782474656201);  // ln(T/300)
-  b.arrC = F(4.67e-12) * m_exp(F(-0.6) * lT300);
-  b.kCpH2 = F(4.0e-16) * m_exp(F(-0.2) * lT300);
-  b.xMH_T = m_exp(F(0.345) * lT300) * F(2041.2414523193154);  // 1/sqrt(2.4e-7 (T/300)^-0.69)
-  b.xe_hot = xe_hot_of(c, b.lnT * F(0.43429448190325176));  // at log10 T
-  b.wdH3T = F(WDH3) * m_exp(F(WDH4) * b.lnT);
-  b.wdHex = F(-WDH5) - F(WDH6) * b.lnT;
-  b.wdC3T = F(WDC3) * m_exp(F(WDC4) * b.lnT);
-  b.wdCex = F(-WDC5) - F(WDC6) * b.lnT;
+  F lT4 = b.lnT - K(9.210340371976184);  // ln(T/1e4)
+  b.arr = K(2.54e-13) * m_exp((K(-0.8163) - K(0.0208) * lT4) * lT4);
+  b.kci = K(5.85e-11) * b.sqT * m_exp(K(-157809.1) * invT) / (K(1) + b.sqT * K(0.003162277660168379));
+  b.kcdH = K(6.67e-12) * b.sqT * m_exp(K(-1) - K(63593.0) * invT);
+  b.kcdH2 = K(5.996e-30) * m_exp(K(4.1881) * b.lnT - K(54657.4) * invT - K(5.6881) * m_log(K(1) + K(6.761e-6) * T));
+  F lT300 = b.lnT - K(5.703782474656201);  // ln(T/300)
+  b.arrC = K(4.67e-12) * m_exp(K(-0.6) * lT300);
+  b.kCpH2 = K(4.0e-16) * m_exp(K(-0.2) * lT300);
+  b.xMH_T = m_exp(K(0.345) * lT300) * K(2041.2414523193154);  // 1/sqrt(2.4e-7 (T/300)^-0.69)
+  b.xe_hot = xe_hot_of(c, b.lnT * K(0.43429448190325176));  // at log10 T
+  b.wdH3T = K(WDH3) * m_exp(K(WDH4) * b.lnT);
+  b.wdHex = K(-WDH5) - K(WDH6) * b.lnT;
+  b.wdC3T = K(WDC3) * m_exp(K(WDC4) * b.lnT);
+  b.wdCex = K(-WDC5) - K(WDC6) * b.lnT;
   return b;
 }
 
@@ -320,86 +326,91 @@ template <class F> struct CoolT {
 // Ly-alpha (Eq. e:k_lya): E_21 5.31e-8 T4^0.15 / (1 + (T4/5)^0.65) exp(-11.84/T4) with
 // E_21/k_B = 1.184e5 K, from ln(T/1e4) and 1e4/T.
 template <class F> TCG_FN F lya_of(F lT4, F invT4) {
-  return F(1.184e5 * KB * 5.31e-8) * m_exp(F(0.15) * lT4 - F(11.84) * invT4) /
-         (F(1) + m_exp(F(0.65) * (lT4 - F(1.6094379124341003))));
+  using K = typename ConstOf<F>::type;
+  return K(1.184e5 * KB * 5.31e-8) * m_exp(K(0.15) * lT4 - K(11.84) * invT4) /
+         (K(1) + m_exp(K(0.65) * (lT4 - K(1.6094379124341003))));
 }
 // free-free Gaunt factor at log10 T = lt
 template <class F> TCG_FN F gff_of(F lt) {
-  F dg = F(5.5) - lt;
-  return F(1.1) + F(0.34) * m_exp(-dg * dg * F(1.0 / 3.0));
+  using K = typename ConstOf<F>::type;
+  F dg = K(5.5) - lt;
+  return K(1.1) + K(0.34) * m_exp(-dg * dg * K(1.0 / 3.0));
 }
 // H2 ro-vibrational LTE rate per molecule from ln(T/1000) and 1000/T (T clamped to
 // [10, 1e4] K by the caller): rotational and vibrational parts
 template <class F> TCG_FN F rovib_lte_of(F lT3, F iT3) {
-  F q = F(0.13) * iT3;
-  F Lrot = F(9.5e-22) * m_exp(F(3.76) * lT3 - q * q * q) / (F(1) + F(0.12) * m_exp(F(2.1) * lT3)) +
-           F(3e-24) * m_exp(F(-0.51) * iT3);
-  F Lvib = F(6.7e-19) * m_exp(F(-5.86) * iT3) + F(1.6e-18) * m_exp(F(-11.7) * iT3);
+  using K = typename ConstOf<F>::type;
+  F q = K(0.13) * iT3;
+  F Lrot = K(9.5e-22) * m_exp(K(3.76) * lT3 - q * q * q) / (K(1) + K(0.12) * m_exp(K(2.1) * lT3)) +
+           K(3e-24) * m_exp(K(-0.51) * iT3);
+  F Lvib = K(6.7e-19) * m_exp(K(-5.86) * iT3) + K(1.6e-18) * m_exp(K(-11.7) * iT3);
   return Lrot + Lvib;
 }
 // CIE cooling of He and metals (before the S weighting) at log10 T = lt
 template <class F, class FC> TCG_FN F cie_of(const CellC<FC>& c, F lt) {
-  F z1 = (lt - F(5.0)) * F(1.0 / 0.15), z2 = (lt - F(5.35)) * F(1.0 / 0.28), z3 = (lt - F(6.3)) * F(1.0 / 0.35);
-  return F(2.0e-23) * m_exp(F(-0.5) * z1 * z1) +
-         c.Zg * (F(5.4e-22) * m_exp(F(-0.5) * z2 * z2) + F(5.0e-23) * m_exp(F(-0.5) * z3 * z3));
+  using K = typename ConstOf<F>::type;
+  F z1 = (lt - K(5.0)) * K(1.0 / 0.15), z2 = (lt - K(5.35)) * K(1.0 / 0.28), z3 = (lt - K(6.3)) * K(1.0 / 0.35);
+  return K(2.0e-23) * m_exp(K(-0.5) * z1 * z1) +
+         c.Zg * (K(5.4e-22) * m_exp(K(-0.5) * z2 * z2) + K(5.0e-23) * m_exp(K(-0.5) * z3 * z3));
 }
 
 template <class F, class FC> TCG_BIG CoolT<F> cool_T(const CellC<FC>& c, const ChemT<F>& b, unsigned flags) {
   TCG_COUNT(cool_T);
+  using K = typename ConstOf<F>::type;
   CoolT<F> k;
   const F T = b.T, lnT = b.lnT;
   const F invT = b.invT;
-  k.fcA = F(1.0e-12) * b.sqT * m_exp(F(-1000.0) * invT);
-  k.fcB = F(1.4e-12) * b.sqT * m_exp(F(-18100.0) / (T + F(1200.0)));
-  k.eps_num = F(5.22) + F(2.25) * m_exp(F(0.147) * lnT);
-  F lT4 = lnT - F(9.210340371976184);
-  F invT4 = F(1e4) * invT;
+  k.fcA = K(1.0e-12) * b.sqT * m_exp(K(-1000.0) * invT);
+  k.fcB = K(1.4e-12) * b.sqT * m_exp(K(-18100.0) / (T + K(1200.0)));
+  k.eps_num = K(5.22) + K(2.25) * m_exp(K(0.147) * lnT);
+  F lT4 = lnT - K(9.210340371976184);
+  F invT4 = K(1e4) * invT;
   k.lyaE = lya_of(lT4, invT4);
-  F lt = lnT * F(0.43429448190325176);
-  k.ffrr = F(1.42e-27) * b.sqT * gff_of(lt) + b.arr * F(KB) * T * (F(0.684) - F(0.0416) * lT4);
+  F lt = lnT * K(0.43429448190325176);
+  k.ffrr = K(1.42e-27) * b.sqT * gff_of(lt) + b.arr * K(KB) * T * (K(0.684) - K(0.0416) * lT4);
   // C+ 158 um: n_e,crit = 53 T4^1/2, n_H,crit = 3e3 T2^(-0.1281 - 0.0087 ln T2), A = 2.3e-6
-  F lT2 = lnT - F(4.605170185988092);
-  k.cpke = F(2.3e-6 / 53.0 * 100.0) * b.sqT * invT;  // / (53 T^1/2 / 100)
-  k.cpkH = F(2.3e-6 / 3e3) * m_exp((F(0.1281) + F(0.0087) * lT2) * lT2);
-  k.cpb = F(2) * m_exp(F(-91.25) * invT);
+  F lT2 = lnT - K(4.605170185988092);
+  k.cpke = K(2.3e-6 / 53.0 * 100.0) * b.sqT * invT;  // / (53 T^1/2 / 100)
+  k.cpkH = K(2.3e-6 / 3e3) * m_exp((K(0.1281) + K(0.0087) * lT2) * lT2);
+  k.cpb = K(2) * m_exp(K(-91.25) * invT);
   // O 3-level: n_crit(T) through 2.5e5 (10 K) and 4.9e4 (5000 K); C: 620 and 150
-  F lT10 = lnT - F(2.302585092994046);
-  const F sO = F(-0.2622274154608984);  // ln(4.9e4/2.5e5)/ln 500
-  const F sC = F(-0.22834652828762741);  // ln(150/620)/ln 500
-  k.ok10 = F(8.91e-5 / 2.5e5) * m_exp(-sO * lT10);
+  F lT10 = lnT - K(2.302585092994046);
+  const F sO = K(-0.2622274154608984);  // ln(4.9e4/2.5e5)/ln 500
+  const F sC = K(-0.22834652828762741);  // ln(150/620)/ln 500
+  k.ok10 = K(8.91e-5 / 2.5e5) * m_exp(-sO * lT10);
   // exp(-E2/T) = exp(-E1/T) exp(-(E2 - E1)/T): two exponentials for the three factors
-  F eO1 = m_exp(F(-227.7) * invT), eO21 = m_exp(F(-(326.6 - 227.7)) * invT);
-  k.ob1 = F(3.0 / 5.0) * eO1;
-  k.ob2 = F(1.0 / 5.0) * (eO1 * eO21);
-  k.ob21 = F(1.0 / 3.0) * eO21;
-  k.ck10 = F(7.93e-8 / 620.0) * m_exp(-sC * lT10);
-  F eC1 = m_exp(F(-23.6) * invT), eC21 = m_exp(F(-(62.4 - 23.6)) * invT);
-  k.cb1 = F(3.0) * eC1;
-  k.cb2 = F(5.0) * (eC1 * eC21);
-  k.cb21 = F(5.0 / 3.0) * eC21;
+  F eO1 = m_exp(K(-227.7) * invT), eO21 = m_exp(K(-(326.6 - 227.7)) * invT);
+  k.ob1 = K(3.0 / 5.0) * eO1;
+  k.ob2 = K(1.0 / 5.0) * (eO1 * eO21);
+  k.ob21 = K(1.0 / 3.0) * eO21;
+  k.ck10 = K(7.93e-8 / 620.0) * m_exp(-sC * lT10);
+  F eC1 = m_exp(K(-23.6) * invT), eC21 = m_exp(K(-(62.4 - 23.6)) * invT);
+  k.cb1 = K(3.0) * eC1;
+  k.cb2 = K(5.0) * (eC1 * eC21);
+  k.cb21 = K(5.0 / 3.0) * eC21;
   // H2 ro-vibrational: T clamped to [10, 1e4] K (equivalently ln T clamped)
   if (flags & FL_NO_ROVIB) {
-    k.rvLlow = F(0); k.rvLLTE = F(1);
+    k.rvLlow = K(0); k.rvLLTE = K(1);
   } else {
-    F lnTc = m_min(m_max(lnT, F(2.302585092994046)), F(9.210340371976184));
-    F x = lnTc * F(0.43429448190325176);
-    F poly = F(-103.0) + x * (F(97.59) + x * (F(-48.05) + x * (F(10.80) + x * F(-0.9032))));
-    k.rvLlow = m_exp(poly * F(LN10));
-    F lT3 = lnTc - F(6.907755278982137);
-    F iT3 = F(1000) / m_min(m_max(T, F(10)), F(1e4));  // 1/T3 = exp(-lT3)
+    F lnTc = m_min(m_max(lnT, K(2.302585092994046)), K(9.210340371976184));
+    F x = lnTc * K(0.43429448190325176);
+    F poly = K(-103.0) + x * (K(97.59) + x * (K(-48.05) + x * (K(10.80) + x * K(-0.9032))));
+    k.rvLlow = m_exp(poly * K(LN10));
+    F lT3 = lnTc - K(6.907755278982137);
+    F iT3 = K(1000) / m_min(m_max(T, K(10)), K(1e4));  // 1/T3 = exp(-lT3)
     k.rvLLTE = rovib_lte_of(lT3, iT3);
   }
-  F st10 = m_sqrt(T * F(0.1));
-  k.coA = F(4e-27) * (T * F(0.1)) * st10;
-  k.coN = F(3e3) * st10;
-  k.grT = F(4.65e-30) * m_exp(F(0.94) * lnT);
-  k.grB = F(0.74) * m_exp(F(-0.068) * lnT);
-  F poly = F(6.92e-1) + lT4 * (F(-5.86e-1) + lT4 * (F(8.16e-1) + lT4 * (F(-5.05e-1) +
-           lT4 * (F(1.18e-1) + lT4 * (F(7.66e-3) + lT4 * F(-5.08e-3))))));
-  k.nebT = F(3.68e-23) * m_exp(poly * F(LN10) - F(3.86) * invT4 - F(0.5) * lT4);
-  k.nebX = F(0.38) - F(0.12) * lT4;
+  F st10 = m_sqrt(T * K(0.1));
+  k.coA = K(4e-27) * (T * K(0.1)) * st10;
+  k.coN = K(3e3) * st10;
+  k.grT = K(4.65e-30) * m_exp(K(0.94) * lnT);
+  k.grB = K(0.74) * m_exp(K(-0.068) * lnT);
+  F poly = K(6.92e-1) + lT4 * (K(-5.86e-1) + lT4 * (K(8.16e-1) + lT4 * (K(-5.05e-1) +
+           lT4 * (K(1.18e-1) + lT4 * (K(7.66e-3) + lT4 * K(-5.08e-3))))));
+  k.nebT = K(3.68e-23) * m_exp(poly * K(LN10) - K(3.86) * invT4 - K(0.5) * lT4);
+  k.nebX = K(0.38) - K(0.12) * lT4;
   if (flags & FL_NO_CIE) {
-    k.cie = F(0);
+    k.cie = K(0);
   } else {
     k.cie = cie_of(c, lt);
   }
@@ -649,21 +660,23 @@ template <class F> struct HRate {
 // when x_H+ -> 1 or x_H2 -> 1/2.
 template <class F, class FC> TCG_FN HRate<F> h_rates(const CellC<FC>& c, const ChemT<F>& b, F xH2, F xH,
                                                                F xe, F lpsi) {
+  using K = typename ConstOf<F>::type;
   HRate<F> r;
-  F zcrH2 = F(2) * c.xi * (F(2.3) * xH2 + F(1.5) * xH);        // Eq. eq:H2_cr
+  F zcrH2 = K(2) * c.xi * (K(2.3) * xH2 + K(1.5) * xH);        // Eq. eq:H2_cr
   F zcd = c.n * (b.kcdH * xH + b.kcdH2 * xH2);
   F ne = xe * c.n;
-  F agrH = F(1e-14 * WDH0) * c.Zd /
-           (F(1) + F(WDH1) * m_exp(F(WDH2) * lpsi) * (F(1) + b.wdH3T * m_exp(b.wdHex * lpsi)));
+  F agrH = K(1e-14 * WDH0) * c.Zd /
+           (K(1) + K(WDH1) * m_exp(K(WDH2) * lpsi) * (K(1) + b.wdH3T * m_exp(b.wdHex * lpsi)));
   r.kn = b.kgr * c.n;
-  r.DH2 = F(1.65) * zcrH2 + c.zpd + c.zpiH2 + zcd;
-  r.I = c.zpiH + F(0.5) * zcrH2 + b.kci * ne;
+  r.DH2 = K(1.65) * zcrH2 + c.zpd + c.zpiH2 + zcd;
+  r.I = c.zpiH + K(0.5) * zcrH2 + b.kci * ne;
   r.Rr = b.arr * ne + agrH * c.n;
   return r;
 }
 
 template <class F, class FC> TCG_FN F log_psi(const CellC<FC>& c, const ChemT<F>& b, F xe) {
-  return m_log(c.G0 * b.sqT / m_max(xe * c.n, F(1e-30)) + F(50));
+  using K = typename ConstOf<F>::type;
+  return m_log(c.G0 * b.sqT / m_max(xe * c.n, K(1e-30)) + K(50));
 }
 
 // ------------------------------------------------------------------ net source terms
@@ -683,6 +696,7 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
                                                             F xH2, F xHp, F xH, const Equil<F>& q, F Td_fixed,
                                                             F Td_guess) {
   TCG_COUNT(source);
+  using K = typename ConstOf<F>::type;
   Src<F> s;
   const F n = c.n;
   const F xe = q.xe;
@@ -695,18 +709,18 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
   s.CH2 = s.form - s.dest;
   s.CHp = s.ion - s.rec;
   // --- heating per H
-  F eps = k.eps_num / (F(1) + F(0.04996) * m_exp(F(0.431) * lp) * (F(1) + F(0.00430) * m_exp(F(0.692) * lp)));
-  F qH = (F(7.5) + F(24.5) * m_sqrt(xe / (xe + F(0.07)))) * F(EV);
+  F eps = k.eps_num / (K(1) + K(0.04996) * m_exp(K(0.431) * lp) * (K(1) + K(0.00430) * m_exp(K(0.692) * lp)));
+  F qH = (K(7.5) + K(24.5) * m_sqrt(xe / (xe + K(0.07)))) * K(EV);
   F dcol = n * (xH * k.fcA + xH2 * k.fcB);
-  F fcol = dcol / (dcol + F(2e-7) + c.zpd);
-  F G = F(1e-26) * c.G0 * eps * c.Zd                                  // photoelectric
-      + c.xi * (xH * qH + F(2) * xH2 * c.qH2)                           // cosmic rays
-      + xH * F(3.4 * EV) * c.zpiH + xH2 * F(4.4 * EV) * c.zpiH2         // photoionisation
-      + r.kn * xH * (F(0.2 * EV) + F(4.2 * EV) * fcol)                  // H2 formation
-      + c.zpd * xH2 * (F(16.0 * EV) * fcol + F(0.4 * EV));             // UV pumping + dissociation
+  F fcol = dcol / (dcol + K(2e-7) + c.zpd);
+  F G = K(1e-26) * c.G0 * eps * c.Zd                                  // photoelectric
+      + c.xi * (xH * qH + K(2) * xH2 * c.qH2)                           // cosmic rays
+      + xH * K(3.4 * EV) * c.zpiH + xH2 * K(4.4 * EV) * c.zpiH2         // photoionisation
+      + r.kn * xH * (K(0.2 * EV) + K(4.2 * EV) * fcol)                  // H2 formation
+      + c.zpd * xH2 * (K(16.0 * EV) * fcol + K(0.4 * EV));             // UV pumping + dissociation
   // --- cooling per n^2
-  F Lhyd = xH * xe * (k.lyaE + F(13.6 * EV) * b.kci)                  // Ly-alpha + coll. ionisation
-         + F(4.48 * EV) * xH2 * (xH * b.kcdH + xH2 * b.kcdH2)          // coll. dissociation
+  F Lhyd = xH * xe * (k.lyaE + K(13.6 * EV) * b.kci)                  // Ly-alpha + coll. ionisation
+         + K(4.48 * EV) * xH2 * (xH * b.kcdH + xH2 * b.kcdH2)          // coll. dissociation
          + k.ffrr * xe * xHp;                                           // free-free + recombination
   {
     F nL = n * k.rvLlow;                                                // H2 ro-vibrational
@@ -717,59 +731,59 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
     F Lrv;
     if constexpr (Prec<F>::fp32_range) Lrv = k.rvLLTE * (nL / den);
     else Lrv = k.rvLLTE * nL / den;
-    Lhyd += (den > F(0)) ? xH2 * Lrv / n : F(0);
+    Lhyd += (den > K(0)) ? xH2 * Lrv / n : K(0);
   }
   F Lmet;
   {
     // C+ two-level
-    F C10 = n * (k.cpke * xe + k.cpkH * (xH + F(0.5) * xH2));
+    F C10 = n * (k.cpke * xe + k.cpkH * (xH + K(0.5) * xH2));
     F C01 = C10 * k.cpb;
     // (energies in K; k_B and 1/n applied once at the end, which keeps the partial
     // sums far above FP32's smallest normal number)
-    F lines = q.xCp * (C01 / (F(2.3e-6) + C10 + C01)) * F(2.3e-6 * 91.25);
+    F lines = q.xCp * (C01 / (K(2.3e-6) + C10 + C01)) * K(2.3e-6 * 91.25);
     // O and C three-level atoms, H and H2 collisions (H2 at half the H rate).  The level
     // populations relative to the ground state are r1 = p1/det and r2 = p2/det, and the
     // cooling per atom (r1 A1 E1 + r2 (A20 E2 + A21 E21)) / (1 + r1 + r2) is taken as
     // (p1 A1 E1 + p2 (...)) / (det + p1 + p2), one quotient instead of three.
-    F coll = n * (xH + F(0.5) * xH2);
+    F coll = n * (xH + K(0.5) * xH2);
     {
       F C10o = k.ok10 * coll;
       F C01o = C10o * k.ob1, C02o = C10o * k.ob2, C12o = C10o * k.ob21;
-      F a11 = F(8.91e-5) + C10o + C12o;
-      F bb = F(1.75e-5) + C10o;
-      F a22 = F(1.34e-10) + F(1.75e-5) + F(2) * C10o;
+      F a11 = K(8.91e-5) + C10o + C12o;
+      F bb = K(1.75e-5) + C10o;
+      F a22 = K(1.34e-10) + K(1.75e-5) + K(2) * C10o;
       F det = a11 * a22 - bb * C12o;
       F p1 = C01o * a22 + bb * C02o;
       F p2 = a11 * C02o + C12o * C01o;
-      lines += q.xO * (p1 * F(8.91e-5 * 227.7) + p2 * F(1.34e-10 * 326.6 + 1.75e-5 * (326.6 - 227.7))) /
+      lines += q.xO * (p1 * K(8.91e-5 * 227.7) + p2 * K(1.34e-10 * 326.6 + 1.75e-5 * (326.6 - 227.7))) /
                (det + p1 + p2);
     }
     {
       F C10c = k.ck10 * coll;
       F C01c = C10c * k.cb1, C02c = C10c * k.cb2, C12c = C10c * k.cb21;
-      F a11 = F(7.93e-8) + C10c + C12c;
-      F bb = F(2.65e-7) + C10c;
-      F a22 = F(2.0e-14) + F(2.65e-7) + F(2) * C10c;
+      F a11 = K(7.93e-8) + C10c + C12c;
+      F bb = K(2.65e-7) + C10c;
+      F a22 = K(2.0e-14) + K(2.65e-7) + K(2) * C10c;
       F det = a11 * a22 - bb * C12c;
       F p1 = C01c * a22 + bb * C02c;
       F p2 = a11 * C02c + C12c * C01c;
-      lines += q.xC * (p1 * F(7.93e-8 * 23.6) + p2 * F(2.0e-14 * 62.4 + 2.65e-7 * (62.4 - 23.6))) /
+      lines += q.xC * (p1 * K(7.93e-8 * 23.6) + p2 * K(2.0e-14 * 62.4 + 2.65e-7 * (62.4 - 23.6))) /
                (det + p1 + p2);
     }
-    Lmet = lines * F(KB) / n;
+    Lmet = lines * K(KB) / n;
     // CO (stand-in with LVG-like trapping)
-    Lmet += q.xCO * k.coA / (F(1) + n / k.coN + q.xCO * c.NtX * F(1e-17));
+    Lmet += q.xCO * k.coA / (K(1) + n / k.coN + q.xCO * c.NtX * K(1e-17));
     // grain-assisted recombination
     Lmet += k.grT * m_exp(k.grB * lp) * xe * c.Zd;
     // nebular lines (Eq. e:Lambda_neb)
-    F ne2 = xe * n * F(0.01);
-    Lmet += c.Zg * xe * xHp * k.nebT / (F(1) + F(0.12) * m_exp(k.nebX * m_log(ne2)));
+    F ne2 = xe * n * K(0.01);
+    Lmet += c.Zg * xe * xHp * k.nebT / (K(1) + K(0.12) * m_exp(k.nebX * m_log(ne2)));
     // gas-dust (Eq. eq:gas-dust)
     if constexpr (Prec<F>::cls == 3) s.Td = Td_fixed;  // derivatives: the caller has differentiated the root
-    else s.Td = (Td_fixed > F(0)) ? Td_fixed : dust_T(c, b.T, b.sqT, Td_guess);
-    Lmet += F(3.2e-34) * b.sqT * (b.T - s.Td) * c.Zd;
+    else s.Td = (Td_fixed > K(0)) ? Td_fixed : dust_T(c, b.T, b.sqT, Td_guess);
+    Lmet += K(3.2e-34) * b.sqT * (b.T - s.Td) * c.Zd;
   }
-  F L = Lhyd + (F(1) - b.S) * Lmet + b.S * k.cie;
+  F L = Lhyd + (K(1) - b.S) * Lmet + b.S * k.cie;
   s.G = G;
   s.L = L;
   s.H = n * G - n * n * L;
