@@ -119,10 +119,13 @@ TCG_FN dualf m_max(dualf a, float b) { return (a.v < b) ? dualf::make(b, 0.0f) :
 TCG_FN dualf m_min(dualf a, float b) { return (b < a.v) ? dualf::make(b, 0.0f) : a; }
 TCG_FN dualf m_abs(dualf a) { return (a.v < 0.0f) ? -a : a; }
 
-// The C/O/e equilibrium along one direction, given its root x_e.  With g(x; y) the
-// electron balance's residual, dx_e = -(dg/dy) / (dg/dx): one evaluation of x_C+ at the
-// fixed x_e, its derivative along y by duals and along x by the formula of equilibrium().
-TCG_FN Equil<dualf> equil_tangent(const CellC<float>& c, const ChemT<dualf>& b, dualf xH2, dualf xHp, float xe) {
+// The C/O/e equilibrium along one direction at x_e.  With g(x; y) the electron balance's
+// residual, dx_e = -(dg/dy) / (dg/dx): one evaluation of x_C+ at the fixed x_e, its
+// derivative along y by duals and along x by the formula of equilibrium().  With `refine`,
+// x_e is an estimate: it takes one Newton step, and x_C+ and ln psi move with it to first
+// order.
+TCG_FN Equil<dualf> equil_tangent(const CellC<float>& c, const ChemT<dualf>& b, dualf xH2, dualf xHp, float xe,
+                                  bool refine) {
   TCG_COUNT_T(equil, dualf);
   Equil<dualf> q;
   const dualf w = 1.0f - b.S;
@@ -131,6 +134,8 @@ TCG_FN Equil<dualf> equil_tangent(const CellC<float>& c, const ChemT<dualf>& b, 
   const dualf a0 = w * (xHp + q.xOp + q.xMHp) + b.S * (xHp + b.xe_hot);
   const dualf src = (c.zpiC_rad + c.zcrC) + (1040.0f * c.xi) * xH2;
   const dualf sink0 = src + c.n * (b.kCpH2 * xH2);
+  const bool coupled = w.v * c.xCtot > 0.0f && src.v > 0.0f;
+  if (refine) xe = coupled ? fminf(fmaxf(xe, a0.v), a0.v + w.v * c.xCtot) : a0.v;
   const float ne = fmaxf(xe * c.n, 1e-30f);
   const dualf psi = (c.G0 * dual_rcp(ne)) * b.sqT + 50.0f;
   const dualf lp = m_log(psi);
@@ -145,11 +150,12 @@ TCG_FN Equil<dualf> equil_tangent(const CellC<float>& c, const ChemT<dualf>& b, 
   const float dD = float(WDC1) * (float(WDC2) * pa.v * (1.0f + pb.v) + pa.v * b.wdCex.v * pb.v) * dlp;
   const float dagr = -agr.v * dual_rcp(D.v) * dD;
   const float dr = -r.v * dual_rcp(den.v) * ((dagr + b.arrC.v) * c.n);
-  const bool coupled = w.v * c.xCtot > 0.0f && src.v > 0.0f;
-  const float dxe = coupled ? (a0.d + w.d * r.v + w.v * r.d) * dual_rcp(1.0f - w.v * dr) : a0.d;
-  q.xe = dualf::make(xe, dxe);
-  q.xCp = dualf::make(r.v, r.d + dr * dxe);
-  q.lpsi = dualf::make(lp.v, lp.d + dlp * dxe);
+  const float igp = dual_rcp(1.0f - w.v * dr);
+  const float dxe = coupled ? (a0.d + w.d * r.v + w.v * r.d) * igp : a0.d;
+  const float sx = (refine && coupled) ? (a0.v + w.v * r.v - xe) * igp : 0.0f;
+  q.xe = dualf::make(xe + sx, dxe);
+  q.xCp = dualf::make(fminf(fmaxf(r.v + dr * sx, 0.0f), c.xCtot), r.d + dr * dxe);
+  q.lpsi = dualf::make(lp.v + dlp * sx, lp.d + dlp * dxe);
   const dualf fr = m_max((c.xCtot > 0.0f) ? q.xCp / c.xCtot : dualf(0.0), xHp);
   q.xCO = (2.0f * c.xCtot) * xH2 * (1.0f - fr) / (1.0f + c.rCO2);
   q.xC = c.xCtot - q.xCp - q.xCO;
@@ -157,25 +163,36 @@ TCG_FN Equil<dualf> equil_tangent(const CellC<float>& c, const ChemT<dualf>& b, 
   return q;
 }
 
-// The dust temperature along one direction, given its root td (the energy balance of
-// dust_T differentiated).
-TCG_FN dualf dust_tangent(const CellC<float>& c, const ChemT<dualf>& b, float td) {
+// The dust temperature along one direction at td (the energy balance of dust_T
+// differentiated); with `refine`, td takes one Newton step first.
+TCG_FN dualf dust_tangent(const CellC<float>& c, const ChemT<dualf>& b, float td, bool refine) {
   if (!(c.Zd > 0.0f)) return b.T;
   const dualf C = c.Cgd * b.sqT;
-  const float y2 = td * td;
-  const float dh = c.Bd * td * (6.0f * y2 * y2 - 2.0f * c.Tc4) + C.v;
+  float y2 = td * td;
+  float dh = c.Bd * td * (6.0f * y2 * y2 - 2.0f * c.Tc4) + C.v;
+  if (refine) {
+    td -= (c.Bd * y2 * (y2 * y2 - c.Tc4) - c.Gd - C.v * (b.T.v - td)) * dual_rcp(dh);
+    y2 = td * td;
+    dh = c.Bd * td * (6.0f * y2 * y2 - 2.0f * c.Tc4) + C.v;
+  }
   return dualf::make(td, (C.d * (b.T.v - td) + C.v * b.T.d) * dual_rcp(dh));
 }
 
-// Derivatives of f = (H/K, C_H2, C_H+) and of (x_e, x_C+, x_CO) along ln T, x_H2 and x_H+
-// at one state, given its x_e and dust temperature: df[i][j] and dq[i][j], j the
-// direction, for the directions j0 <= j < j1.  The temperature blocks are differentiated
-// once; the two abundance directions run on them with their derivatives cleared.  `hk` is
-// 1 / (mu_H k_B / (gamma - 1)): H/K = (Gamma - n Lambda) hk stays in FP32's range at any
-// density.
+// f = (H/K, C_H2, C_H+) in FP32 with the estimates of x_e and T_d refined, and T_d's
+// derivatives (the outputs of source_tangents beyond the Jacobian).
+struct Tan32 {
+  float f[3], xe, td, dtd[3];
+};
+
+// Derivatives of f and of (x_e, x_C+, x_CO) along ln T, x_H2 and x_H+ at one state, given
+// its x_e and dust temperature: df[i][j] and dq[i][j], j the direction, for the directions
+// j0 <= j < j1.  The temperature blocks are differentiated once; the two abundance
+// directions run on them with their derivatives cleared.  `hk` is 1 / (mu_H k_B / (gamma -
+// 1)): H/K = (Gamma - n Lambda) hk stays in FP32's range at any density.  With `val`, x_e and
+// td are estimates (one Newton step each) and the values are returned too.
 TCG_BIG inline void source_tangents(const CellC<float>& c, unsigned flags, float hk, float T, float x2, float xp,
                                     float xH, float xe, float td, float (*df)[3], float (*dq)[3], int j0 = 0,
-                                    int j1 = 3) {
+                                    int j1 = 3, Tan32* val = nullptr) {
   ChemT<dualf> b = chem_T(c, dualf::make(T, (j0 == 0) ? T : 0.0f), flags);
   CoolT<dualf> k = cool_T(c, b, flags);
 #pragma unroll 1
@@ -188,14 +205,22 @@ TCG_BIG inline void source_tangents(const CellC<float>& c, unsigned flags, float
     }
     const dualf X2 = dualf::make(x2, (j == 1) ? 1.0f : 0.0f), XP = dualf::make(xp, (j == 2) ? 1.0f : 0.0f);
     const dualf XH = dualf::make(xH, (j == 0) ? 0.0f : (j == 1) ? -2.0f : -1.0f);
-    const Equil<dualf> q = equil_tangent(c, b, X2, XP, xe);
-    const Src<dualf> s = source(c, b, k, X2, XP, XH, q, dust_tangent(c, b, td), dualf(-1.0));
+    const Equil<dualf> q = equil_tangent(c, b, X2, XP, xe, val != nullptr);
+    const Src<dualf> s = source(c, b, k, X2, XP, XH, q, dust_tangent(c, b, td, val != nullptr), dualf(-1.0));
     df[0][j] = (s.G.d - c.n * s.L.d) * hk;
     df[1][j] = s.CH2.d;
     df[2][j] = s.CHp.d;
     dq[0][j] = q.xe.d;
     dq[1][j] = q.xCp.d;
     dq[2][j] = q.xCO.d;
+    if (val) {
+      val->f[0] = (s.G.v - c.n * s.L.v) * hk;
+      val->f[1] = s.CH2.v;
+      val->f[2] = s.CHp.v;
+      val->xe = q.xe.v;
+      val->td = s.Td.v;
+      val->dtd[j] = s.Td.d;
+    }
   }
 }
 

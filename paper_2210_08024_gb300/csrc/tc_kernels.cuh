@@ -526,69 +526,154 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
   CHp = double(sr.ion) - double(sr.rec);
 }
 
-// Newton with the Jacobian from FP32 dual numbers (source_tangents): the fast path of
-// the FP64 solve.  Each iteration evaluates f once, in FP64, where the forward
-// differences of newton_iter take three more evaluations; the first iteration takes f
-// from the substep start's source terms `src` = (H, C_H2, C_H+), so it evaluates nothing
-// (they hold the stored x_e instead of the one at the new mu: the start of the iteration
-// is that much off, its root is not).  The FP32 Jacobian is good to ~1e-6, so steps
-// contract quadratically until there and by ~1e-6 a step from there on.
-//
+// Newton with FP32 dual numbers (source_tangents): the fast path of the FP64 solve, in two
+// phases on the same equations.
+//  1. FP32 Newton from the start state: values and Jacobian from one dual-number evaluation
+//     an iteration, x_e and T_d carried along (predicted by their derivatives, one Newton
+//     step each), until a step is below 3e-5 or stops shrinking at FP32's rounding floor.
+//     This takes the varying part of the iteration counts, which would leave lanes of a
+//     warp waiting, off the FP64 pipe.
+//  2. FP64: f in FP64 at the FP32 root (~1e-6 off), the correction with the FP32 Jacobian of
+//     the last dual-number evaluation (rebuilt at the iterate when a step does not shrink a
+//     thousandfold).  Two evaluations usually do.
 // Converged when every step is below rtol |y_i| as in newton_iter, or one step earlier,
 // when two steps in a row show that the next would lie far below it: with rho = d_k /
-// d_(k-1), what remains after step k is at most ~rho d_k, accepted below 1e-2 rtol
-// (measured on 20,000 slab cells against a 64-bit reference converged to rounding: 2-norm
-// error of T 1.4e-16, of x_e 2.3e-16; the plain iteration 3.9e-15 and 4.7e-14).  The C/O/e equilibrium
-// of the last evaluation is moved along the last step by its derivatives, which leaves
-// less than the step squared (below 1e-16).
+// d_(k-1), what remains after step k is at most ~rho d_k, accepted below 1e-2 rtol (the
+// errors against a 64-bit reference stand at tests/test_tangent.py's bound).  The C/O/e
+// equilibrium of the last evaluation is moved along the last step by its derivatives.
 //
-// Returns the iterations, or -1 when a step would have to be damped, fails to shrink by
-// half after the second iteration or is not finite, or when TAN_MAXIT iterations pass;
-// the plain solver then takes the substep from its start, as if this one had not been
-// tried.  Hard substeps (2% of the random states'
-// iterations, 0.04% of the slab's) thus keep the plain iteration's path, with its damping,
-// predictor and halving decisions.  (Damping here too solved some substeps that the plain
-// iteration halves, which changed the substep grid of 5 in 13,824 cells near x_H = 0.)
+// Returns the iterations of both phases, or -1 when a step would have to be damped, fails to
+// shrink by half or is not finite, or when TAN_MAXIT iterations pass; the plain solver then
+// takes the substep from its start, as if this one had not been tried.  Hard substeps (2% of
+// the random states' iterations, 0.04% of the slab's) thus keep the plain iteration's path,
+// with its damping, predictor and halving decisions.  (Damping here too solved some substeps
+// that the plain iteration halves, which changed the substep grid of 5 in 13,824 cells near
+// x_H = 0.)
 constexpr int TAN_MAXIT = 12;
+constexpr int TAN_MAXIT32 = 8;
 constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
+
+// source_tangents over the cell's lanes: with four, each takes one direction (the last
+// repeats the third) and they exchange.
+template <int LPC>
+TCG_FN void tangents(const CellC<float>& c, unsigned flags, float hk, float T, float x2, float xp, float xH, float xe,
+                     float td, float (*df)[3], float (*dq)[3], Tan32* val = nullptr) {
+  if constexpr (LPC == 4) {
+    const int q = lane_in_cell<4>(), j = (q < 3) ? q : 2;
+    float tf[3][3], tq[3][3];
+    source_tangents(c, flags, hk, T, x2, xp, xH, xe, td, tf, tq, j, j + 1, val);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float vf = (j == 0) ? tf[i][0] : (j == 1) ? tf[i][1] : tf[i][2];
+      const float vq = (j == 0) ? tq[i][0] : (j == 1) ? tq[i][1] : tq[i][2];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        df[i][r] = from_lane<4>(vf, r);
+        dq[i][r] = from_lane<4>(vq, r);
+      }
+    }
+    if (val) {
+      const float vt = (j == 0) ? val->dtd[0] : (j == 1) ? val->dtd[1] : val->dtd[2];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) val->dtd[r] = from_lane<4>(vt, r);
+      // one copy of the values for the whole cell
+#pragma unroll
+      for (int i = 0; i < 3; ++i) val->f[i] = from_lane<4>(val->f[i], 0);
+      val->xe = from_lane<4>(val->xe, 0);
+      val->td = from_lane<4>(val->td, 0);
+    }
+  } else {
+    source_tangents(c, flags, hk, T, x2, xp, xH, xe, td, df, dq, 0, 3, val);
+  }
+}
+
 template <int LPC = 1>
 TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double mu, double Kinv,
-                          const double* yn, double dts, const double* src, double* y, double& xe_g, double& td_g,
-                          Equil<double>* qb) {
-  double f[3] = {src[0] * Kinv, src[1], src[2]};
+                          const double* yn, double dts, double* y, double& xe_g, double& td_g, Equil<double>* qb) {
   const float hk = float(1.0 / (double(c.muH) * KB * 1.5));
+  const float h = float(dts);
+  float df[3][3], dq[3][3], dtd[3];
+  int it32 = 0, res = -1;
+  // Both loops leave through their one end, with a flag, so that the lanes of a warp meet
+  // again there: a return inside let each exit run the second phase on its own.
+  bool ok = true;
+  {  // ---- phase 1, in changes from the start state: T_mu = yn0 (1 + D[0]), x = yn + D
+    const float T0 = float(mu * yn[0]), iy0 = 1.0f / float(yn[0]);
+    const float xn[3] = {0.0f, float(yn[1]), float(yn[2])}, xHn = float(1.0 - 2.0 * yn[1] - yn[2]);
+    float D[3] = {0.0f, 0.0f, 0.0f}, xe = float(xe_g), td = float(td_g), prev = 3e38f;
+    for (;;) {
+      ++it32;
+      const float a = 1.0f + D[0];
+      const float x[3] = {a, fmaxf(xn[1] + D[1], 0.0f), fmaxf(xn[2] + D[2], 0.0f)};
+      const float xH = fmaxf(xHn - 2.0f * D[1] - D[2], 0.0f);
+      Tan32 v;
+      tangents<LPC>(cf, p.flags, hk, T0 * a, x[1], x[2], xH, xe, td, df, dq, &v);
+      float J[3][3], r[3], u[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float s = (i == 0) ? h * iy0 : h;
+        r[i] = s * v.f[i] - D[i];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) J[i][j] = ((i == j) ? x[0] : 0.0f) * ((i == 0) ? 1.0f : 0.0f) - s * df[i][j];
+        if (i > 0) J[i][i] += 1.0f;
+        if (i > 0 && x[i] < float(TAN_TRACE) && fabsf(h * v.f[i]) < float(TAN_TRACE)) {  // left to phase 2
+          r[i] = 0.0f;
+          J[i][0] = J[i][3 - i] = 0.0f;
+        }
+      }
+      ok = solve3<float>(J, r, u);
+      float rel = fabsf(u[0]);
+#pragma unroll
+      for (int i = 1; i < 3; ++i) {
+        if (!(u[i] >= -0.98f * x[i])) {
+          ok = ok && fabsf(u[i]) <= 1e-8f;
+          u[i] = -0.98f * x[i];  // too little to matter to the others; phase 2 settles it
+        }
+        rel = fmaxf(rel, fabsf(u[i]) / (x[i] + u[i] + 1e-8f));
+      }
+      ok = ok && u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * xH && isfinite(rel);
+      if (!ok) break;
+      D[0] += a * u[0];
+      D[1] += u[1];
+      D[2] += u[2];
+      xe = v.xe + dq[0][0] * u[0] + dq[0][1] * u[1] + dq[0][2] * u[2];
+      td = v.td + v.dtd[0] * u[0] + v.dtd[1] * u[1] + v.dtd[2] * u[2];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) dtd[i] = v.dtd[i];
+      if (rel < 3e-5f) break;
+      if (it32 > 2 && !(rel <= 0.5f * prev)) {
+        ok = rel < 1e-3f;  // FP32's rounding floor
+        break;
+      }
+      ok = it32 < TAN_MAXIT32;
+      if (!ok) break;
+      prev = rel;
+    }
+    y[0] = yn[0] + yn[0] * double(D[0]);
+#pragma unroll
+    for (int i = 1; i < 3; ++i) {
+      y[i] = yn[i] + double(D[i]);
+      if (!(y[i] > 0.0)) y[i] = 0.01 * yn[i];
+    }
+    xe_g = double(xe);
+    td_g = double(td);
+  }
+  // ---- phase 2
   float prev = -1.0f;  // size of the previous step, if that was whole
-  const int maxit = (p.newton_max < TAN_MAXIT) ? p.newton_max : TAN_MAXIT;
-  for (int it = 1; it <= maxit; ++it) {
+  bool fresh = false;  // rebuild the Jacobian at the next iterate
+  for (int it = 1; ok && it <= TAN_MAXIT; ++it) {
     TCG_COUNT_D(tangent_it);
-    if (it > 1) {
+    double f[3];
+    {
       ChemT<double> b = chem_T(c, mu * y[0], p.flags);
       CoolT<double> k = cool_T(c, b, p.flags);
       feval64(c, b, k, y[1], y[2], Kinv, xe_g, td_g, f, qb);
     }
     const double xH = 1.0 - 2.0 * y[1] - y[2];
     const float y0 = float(y[0]), x2 = float(y[1]), xp = float(y[2]);
-    float df[3][3], dq[3][3];
-    if constexpr (LPC == 4) {
-      // the cell's lanes take one direction each (the last repeats the third) and exchange
-      const int q = lane_in_cell<4>(), j = (q < 3) ? q : 2;
-      float tf[3][3], tq[3][3];
-      source_tangents(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), tf, tq, j, j + 1);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const float vf = (j == 0) ? tf[i][0] : (j == 1) ? tf[i][1] : tf[i][2];
-        const float vq = (j == 0) ? tq[i][0] : (j == 1) ? tq[i][1] : tq[i][2];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          df[i][r] = from_lane<4>(vf, r);
-          dq[i][r] = from_lane<4>(vq, r);
-        }
-      }
-    } else {
-      source_tangents(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), df, dq);
-    }
+    if (fresh) tangents<LPC>(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), df, dq);
     // rows scaled: (T_mu equation / T_mu, x_H2, x_H+); unknowns (ln T_mu, x_H2, x_H+)
-    const float iy0 = 1.0f / y0, h = float(dts);
+    const float iy0 = 1.0f / y0;
     float J[3][3], r[3], u[3];
     double d[3], rhs[3];
 #pragma unroll
@@ -606,7 +691,7 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
         J[i][0] = J[i][3 - i] = 0.0f;
       }
     }
-    if (!solve3<float>(J, r, u)) return -1;
+    ok = solve3<float>(J, r, u);
     // T_mu, x_H2, x_H+ and x_H must keep 2% of their values (damped_step limits at 1%),
     // except an abundance whose step is below 1e-8 (too little to matter to the others): it
     // may fall to any positive value, and to 1% of its value where the step rounds to less
@@ -624,32 +709,52 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
           d[i] = -0.99 * y[i];
           whole = false;
         }
-      } else if (!(u[i] >= -0.98f * x)) {
-        return -1;
+      } else {
+        ok = ok && u[i] >= -0.98f * x;
       }
       const double yi = y[i] + d[i];
       const float ri = trace ? float(fabs(d[i]) / (fabs(yi) + 1e-300)) : fabsf(u[i]) / (fabsf(float(yi)) + 1e-30f);
       rel = fmaxf(rel, ri);
     }
-    if (!(u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * float(xH)) || !isfinite(rel)) return -1;
+    ok = ok && u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * float(xH) && isfinite(rel);
+    if (!ok) break;
     y[0] += d[0]; y[1] += d[1]; y[2] += d[2];
     if (!whole) {
       prev = -1.0f;
       continue;
     }
+    const double dxe = double(dq[0][0] * u[0] + dq[0][1] * u[1] + dq[0][2] * u[2]);
     const float rtol = float(p.rtol);
-    if (it > 1 && (rel <= rtol || (prev > 0.0f && rel < 1e-2f * prev && rel * (rel / prev) <= 1e-2f * rtol))) {
+    // how far this step's error can be from it: for the first step, from the Jacobian's
+    // distance to the identity (relative units) and its error, 1e-3 of that at most (its
+    // FP32 rounding, and its change over phase 1's last step, 3e-5 times exponents up to 30)
+    float left = (prev > 0.0f) ? rel / prev : 1.0f;
+    if (it == 1) {
+      float nj = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const float si = (i == 0) ? h * iy0 : h / (((i == 1) ? x2 : xp) + 1e-30f);
+        nj = fmaxf(nj, fabsf(si) * (fabsf(df[i][0]) + fabsf(df[i][1]) * x2 + fabsf(df[i][2]) * xp));
+      }
+      left = (nj < 0.5f) ? 2e-3f * nj : 1.0f;
+    }
+    if (rel <= rtol || (left < 1e-2f && rel * left <= 1e-2f * rtol)) {
       // u is at most ~1e-6 here: the change of x_e, x_C+ and x_CO to first order
-      qb->xe += double(dq[0][0] * u[0] + dq[0][1] * u[1] + dq[0][2] * u[2]);
+      qb->xe += dxe;
       qb->xCp += double(dq[1][0] * u[0] + dq[1][1] * u[1] + dq[1][2] * u[2]);
       qb->xCO += double(dq[2][0] * u[0] + dq[2][1] * u[1] + dq[2][2] * u[2]);
       xe_g = qb->xe;
-      return it;
+      res = it32 + it;
+      break;
     }
-    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev)) return -1;
+    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev)) break;
+    fresh = prev > 0.0f && rel > 1e-3f * prev;
     prev = rel;
+    // the next evaluation's inner roots, predicted along the step
+    xe_g += dxe;
+    td_g += double(dtd[0] * u[0] + dtd[1] * u[1] + dtd[2] * u[2]);
   }
-  return -1;
+  return res;
 }
 
 // Accepts the substep's root y: applies the temperature floor, re-solves the C/O/e
@@ -908,7 +1013,7 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
   }
   if (src) {
     double xg = xe_g, tg = td_g;
-    it = newton_tangent<LPC>(c, *cf, p, s.mu, Kinv, yn, dts, src, y, xg, tg, &qb);
+    it = newton_tangent<LPC>(c, *cf, p, s.mu, Kinv, yn, dts, y, xg, tg, &qb);
     if (it >= 0) { xe_g = xg; td_g = tg; }
   }
   if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);

@@ -586,6 +586,9 @@ template <class F> TCG_BIG Equil<F> equilibrium(const CellC<F>& c, const ChemT<F
       x = xn;
       xe = x;
       if (dx <= tol * x || hi - lo <= tol * hi) break;
+      // in FP64 a Newton step below 1e-8 of x has converged: what it leaves is about half its
+      // square (g''/2g' x ~ 1/2), below rounding
+      if (Prec<F>::cls == 0 && newton && dx <= F(1e-8) * x) break;
       // a caller whose guess is within ~1e-7 of the root (the Jacobian's perturbed
       // evaluations, started from the base point's root) stops after newton_max Newton
       // steps: one step from there is already converged to ~1e-14
@@ -639,10 +642,12 @@ template <class F> TCG_FN F dust_T(const CellC<F>& c, F T, F sqT, F guess) {
     if (h > F(0)) hi = y; else lo = y;
     F dh = c.Bd * y * (F(6) * y2 * y2 - F(2) * c.Tc4) + C;
     F yn = y - h / dh;
-    if (!(yn >= lo && yn <= hi)) yn = F(0.5) * (lo + hi);  // bracket ends allowed, as above
+    const bool newton = (yn >= lo && yn <= hi);  // bracket ends allowed, as above
+    if (!newton) yn = F(0.5) * (lo + hi);
     F dy = m_abs(yn - y);
     y = yn;
     if (dy <= tol * y || hi - lo <= tol * hi) break;
+    if (Prec<F>::cls == 0 && newton && dy <= F(3e-9) * y) break;  // leaves ~5/2 of its square
   }
   return y;
 }
