@@ -97,9 +97,9 @@ typedef struct tc_params {
                                   whose four lanes evaluate the four points of each forward-difference
                                   Jacobian at once (tc_step and tc_step_host only; other modes and
                                   tc_step_batch use 1).  0 (default): for TC_MODE_NEWTON_FP64 and
-                                  TC_MODE_MIXED 4 when the cells times 4 fit the cooperative kernel's
-                                  resident lanes at once (launches too small to fill the GPU, whose
-                                  time is the latency of the slowest cells), else 1, unless
+                                  TC_MODE_MIXED 4 on launches too small to fill the GPU, whose time is
+                                  the latency of the slowest cells (up to 64 and 32 cells per SM), else
+                                  1, unless
                                   tc_autotune has recorded a choice for the launch's size class. */
 } tc_params;
 
@@ -177,8 +177,8 @@ typedef struct tc_tune_choice {
 } tc_tune_choice;
 
 /* Autotuner of the step launch.  Times one step of the cells of *f (device pointers, as
- * for tc_step) in every candidate shape -- 32, 64 or 128 threads per block, the occupancy
- * limit or 4 resident blocks per SM, and for modes TC_MODE_NEWTON_FP64 and TC_MODE_MIXED
+ * for tc_step) in every candidate shape -- 32, 64 or 128 threads per block (256 or 512 too for
+ * the mixed modes on launches that fill the GPU), the occupancy limit or 4 resident blocks per SM, and for modes TC_MODE_NEWTON_FP64 and TC_MODE_MIXED
  * one or four lanes per cell (four only when the cooperative kernel holds the cells in
  * at most 8 waves of its resident lanes) -- with CUDA events on `stream`, each candidate
  * once, or three times (fastest kept) when one step takes under 20 ms, and records the fastest

@@ -263,16 +263,45 @@ static int coop_occupancy(int kmode, int block) {
 
 // Launch shape of one step launch: threads per block, grid and lanes per cell.  Explicit
 // tc_params values win; otherwise the shape tc_autotune recorded for the launch's size
-// class; otherwise 128 threads, the occupancy limit, and for modes 1 and 2 four lanes per
-// cell when every cell's four lanes fit the cooperative kernel's resident lanes at once
-// (4096 random states: FP64 Newton 73.1 ms against 108.8 ms with one lane, mixed 43.7
-// against 55.7 ms; the mixed solve builds one FP32 Jacobian per solve and spends most of
-// its time in the df64 polish and substep-start sources, which four lanes do not
-// shorten).  The persistent grid never exceeds the blocks that hold one lane per cell
-// lane.
+// class; otherwise the rules below and the occupancy limit.  The persistent grid never
+// exceeds the blocks that hold every cell at once.
 struct Shape {
-  int grid, block, lpc;
+  int grid, block, lpc, groups;
 };
+// Threads per block where neither the caller nor the autotuner chose.  Launches of few cells
+// take blocks of one warp: they spread over the SMs, and no lane waits for a block's other
+// warps (random states by FP64 Newton, one lane per cell, 32 / 128 threads: 4096 cells 49 / 61
+// ms, 8000 46 / 58; 12,800 curve cells 15.1 / 15.7).  The mixed kernels' large blocks run in
+// step and fetch their code once (tc_kernels.cuh), which pays as soon as the cells fill them.
+// ms at 32 / 128 / 256 / 512 threads: seeded mixed, slab cells: 20k 5.4 / 5.5 / 5.8 / 6.4, 60k
+// 6.8 / 6.4 / 6.6 / 6.6, 150k 10.3 / 9.3 / 8.3 / 9.2, 300k 14.8 / 11.8 / 10.5 / 10.5, 2M 44.4
+// (128) / 36.2 / 33.5; random states: 4k 40 / 44 / 50 / 62, 30k 76 / 58 / 59 / 69, 100k 178 /
+// 155 / 114 / 98.
+static int default_block(int kmode, long long ntotal, int num_sms) {
+  const long long per = ntotal / num_sms;
+  if (per < 112) return 32;
+  if (kmode != 2 && kmode != 3) return tcg::STEP_THREADS;
+  return (per < 600) ? 128 : (per < 1600) ? 256 : 512;
+}
+
+// Whether a launch of modes 1 and 2 takes four lanes per cell: while the cells' warps of
+// eight are at most two (mode 1) or one (mode 2) per SM partition, where latency decides.  ms
+// with four / one: random states mode 1: 500 32 / 43, 4096 37 / 49, 8000 44 / 46; mode 2: 4096
+// 31 / 34, 8000 50 / 37; slab mode 1: 8000 4.5 / 5.4, mode 2: 8000 4.8 / 4.8; 12,800 curve
+// cells, mode 1: 24 / 15.
+static bool default_coop(int kmode, long long ntotal, int num_sms) {
+  return ntotal <= (long long)num_sms * 32 * ((kmode == 1) ? 2 : 1);
+}
+
+// Cells that a warp of the cooperative kernels advances at once: eight, or fewer where that
+// leaves SM partitions without a warp (lanes of one warp wait for one another; random states,
+// mode 1, ms with 8 / 4 / 2 / 1 cells a warp: 500 cells 32 / 27 / 27 / 25, 2000 33 / 30 / 34 / 37,
+// 4096 37 / 40 / 47 / 56).
+static int coop_groups(long long ntotal, int num_sms) {
+  const long long g = (ntotal + 4LL * num_sms - 1) / (4LL * num_sms);
+  return (g < 1) ? 1 : (g > 8) ? 8 : (int)g;
+}
+
 static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal) {
   int b = h->p.block, per_sm = h->p.blocks_per_sm, lpc = h->p.lanes_per_cell;
   const bool coop_ok = (kmode == 1 || kmode == 2) && !batch;
@@ -282,13 +311,16 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
     per_sm = t.blocks_per_sm;
     lpc = t.lanes_per_cell;
   }
-  if (b <= 0) b = 128;
-  if (b > 128) b = 128;  // kernels are compiled with __launch_bounds__(128)
+  const bool auto_block = b <= 0;
+  const int bmax = tcg::step_threads(kmode, 1);  // as the kernels are compiled
+  if (b > bmax) b = bmax;
   b = (b / 32) * 32;
   if (b < 32) b = 32;
   if (!coop_ok) lpc = 1;
-  if (lpc <= 0) lpc = (coop_ok && ntotal * 4 <= (long long)h->num_sms * coop_occupancy(kmode, b) * b) ? 4 : 1;
+  if (lpc <= 0) lpc = (coop_ok && default_coop(kmode, ntotal, h->num_sms)) ? 4 : 1;
   if (lpc != 4) lpc = 1;
+  if (auto_block) b = default_block(kmode, ntotal, h->num_sms);
+  if (lpc == 4 && b > tcg::STEP_THREADS) b = tcg::STEP_THREADS;
   if (per_sm <= 0) {
     per_sm = (lpc == 4) ? coop_occupancy(kmode, b)
              : (kmode == 0) ? tcg::occupancy_mode0_impl(b)
@@ -297,10 +329,11 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
              : (kmode == 3) ? tcg::occupancy_mode3_impl(b) : tcg::occupancy_mode4_impl(b);
   }
   long long g = (long long)h->num_sms * per_sm;
-  long long need = (ntotal * lpc + b - 1) / b;
+  const int groups = (lpc == 4) ? coop_groups(ntotal, h->num_sms) : 32;
+  long long need = ((ntotal + groups - 1) / groups * 32 + b - 1) / b;
   if (g > need) g = need;
   if (g < 1) g = 1;
-  return Shape{(int)g, b, lpc};
+  return Shape{(int)g, b, lpc, groups};
 }
 
 // Grows the cost-ordering workspace to ncell cells (not while `st` is being captured).
@@ -340,6 +373,7 @@ static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long 
   if (cudaMemsetAsync(h->d_cursor, 0, sizeof(unsigned long long), st) != cudaSuccess) return TC_ECUDA;
   tcg::DevParams dp = dev_params(h->p);
   dp.mlp_mma = h->d_mlp_mma;
+  dp.groups = sh.groups;
   // cost-ordered queue: only worth it when the launch holds more cells than a few warps
   if (h->p.order_cells && ntotal > 256 && order_workspace(h, ntotal, st)) {
     if (tcg::launch_order(batch, f, h->d_boxes, dp, dt, ntotal, h->d_okey, h->d_ohist, h->d_order, h->num_sms, st) !=
@@ -418,7 +452,9 @@ int tc_autotune(tc_handle* h, const tc_fields* f, double dt_s, void* stream, tc_
   // most 8 waves of resident lanes (beyond that it is slower by construction)
   const bool coop_ok = (kmode == 1 || kmode == 2) &&
                        (long long)f->ncell * 4 <= 8LL * h->num_sms * coop_occupancy(kmode, 128) * 128;
-  const int blocks[3] = {32, 64, 128};
+  // the mixed kernels' large blocks too, where the cells fill them
+  const int blocks[5] = {32, 64, 128, 256, 512};
+  const int nblk = ((kmode == 2 || kmode == 3) && f->ncell >= 1024LL * h->num_sms) ? 5 : 3;
   const int per_sms[2] = {0, 4};
   const int lpcs[2] = {1, 4};
   // One run in the default shape first (it also sets how often each candidate repeats).
@@ -440,7 +476,7 @@ int tc_autotune(tc_handle* h, const tc_fields* f, double dt_s, void* stream, tc_
   rc = run(&ms0);
   const int reps = (rc == TC_OK && ms0 < 20.f) ? 3 : 1;
   tc_tune_choice bestc = {0, 0, 0, 3.4e38f};
-  for (int ib = 0; ib < 3 && rc == TC_OK; ++ib)
+  for (int ib = 0; ib < nblk && rc == TC_OK; ++ib)
     for (int ip = 0; ip < 2 && rc == TC_OK; ++ip)
       for (int il = 0; il < (coop_ok ? 2 : 1) && rc == TC_OK; ++il) {
         h->p.block = blocks[ib];

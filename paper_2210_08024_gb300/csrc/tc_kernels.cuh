@@ -116,6 +116,17 @@ __device__ __forceinline__ long long claim_cells_lpc(unsigned long long* cursor)
   }
 }
 
+// Where the warps of a block meet, so that they run the same part of the step's code at the
+// same time: the kernels' code (100-200 KB) exceeds the instruction caches, and warps at
+// unrelated places each stream it on their own (fetch stalls are the mixed kernels' largest).
+// Each of a block's four warps sits on another SM partition.
+template <bool SYNC>
+TCG_FN void block_meet() {
+#ifdef __CUDA_ARCH__
+  if constexpr (SYNC) __syncthreads();
+#endif
+}
+
 // Lane-resident state of the cell being advanced.
 struct LaneState {
   double t, Tmu, xH2, xHp, mu;
@@ -1247,32 +1258,42 @@ TCG_FN bool polish_hp(const CellC<F>& c, const DevParams& p, double mu, double K
 // iteration before the polish and the Jacobian.  FP64 work: the Newton updates and
 // residuals, and the fallback.  The solve starts from `seed` when given, else from the
 // start state.
-template <int LPC = 1>
+//
+// SYNC: a block runs the substep in step (block_meet below); every thread calls, those
+// without a substep with need = false.
+template <int LPC = 1, bool SYNC = false>
 TCG_FN void substep_mixed_solve(const CellC<double>& c, const CellC<df64>& cd, const CellC<float>& cf,
                                 const DevParams& p, double dt, double dts, bool last, LaneState& s, float& xe_g,
-                                float& td_g, const df64& td_hp, const double* seed) {
+                                float& td_g, const df64& td_hp, const double* seed, bool need = true) {
   const double yn[3] = {s.Tmu, s.xH2, s.xHp};
   const double Kinv = 1.0 / c.K;
-  double y[3] = {yn[0], yn[1], yn[2]};
-  if (seed) { y[0] = seed[0]; y[1] = seed[1]; y[2] = seed[2]; }
+  double y[3];
   float J[3][3];
-  bool polish = false;
-  int spent = 0;
-  int it = newton_mixed<LPC>(cf, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, J, polish, seed ? SEED_MAXIT : 0, &spent);
-  if (seed) s.status |= (it >= 0) ? ST_SEEDED : ST_SEED_FAIL;
-  if (it < 0 && seed) {
-    // a seed that did not lead to convergence within SEED_MAXIT iterations: start again
-    // from the start state (the abandoned iterations count too)
-    s.iters += spent;
-    y[0] = yn[0]; y[1] = yn[1]; y[2] = yn[2];
-    it = newton_mixed<LPC>(cf, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, J, polish);
+  int it = -1;
+  if (need) {
+    // from the seed when given; a seed that does not lead to convergence within SEED_MAXIT
+    // iterations: once more from the start state (the abandoned iterations count too)
+    bool seeded = seed != nullptr, again;
+    do {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) y[i] = seeded ? seed[i] : yn[i];
+      bool polish = false;
+      int spent = 0;
+      it = newton_mixed<LPC>(cf, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, J, polish, seeded ? SEED_MAXIT : 0, &spent);
+      if (seeded) s.status |= (it >= 0) ? ST_SEEDED : ST_SEED_FAIL;
+      if (it >= 0 && polish) s.status |= ST_POLISH;
+      again = seeded && it < 0;
+      if (again) s.iters += spent;
+      seeded = false;
+    } while (again);
   }
+  block_meet<SYNC>();
+  if (!need) return;
   Equil<df64> qlast;
   const int it32 = it;
   bool have32 = false;
   double y32[3];
   if (it >= 0) {
-    if (polish) s.status |= ST_POLISH;
     y32[0] = y[0]; y32[1] = y[1]; y32[2] = y[2];
     have32 = true;
     fd_jacobian32<LPC>(cf, p, s.mu, Kinv, dts, y, xe_g, td_g, J);
@@ -1308,12 +1329,14 @@ TCG_FN void substep_mixed_solve(const CellC<double>& c, const CellC<df64>& cd, c
   xe_g = float(s.xe);
 }
 
-template <int LPC = 1>
+template <int LPC = 1, bool SYNC = false>
 TCG_FN void substep_mixed(const CellC<double>& c, const CellC<df64>& cd, const CellC<float>& cf, const DevParams& p,
-                          double dt, LaneState& s, float& xe_g, float& td_g, df64& td_hp) {
-  bool last;
-  const double dts = substep_start_t<df64>(cd, c.K, p, dt, s, td_hp, last);
-  substep_mixed_solve<LPC>(c, cd, cf, p, dt, dts, last, s, xe_g, td_g, td_hp, nullptr);
+                          double dt, LaneState& s, float& xe_g, float& td_g, df64& td_hp, bool need = true) {
+  bool last = false;
+  double dts = 0.0;
+  if (need) dts = substep_start_t<df64>(cd, c.K, p, dt, s, td_hp, last);
+  block_meet<SYNC>();
+  substep_mixed_solve<LPC, SYNC>(c, cd, cf, p, dt, dts, last, s, xe_g, td_g, td_hp, nullptr, need);
 }
 
 // ------------------------------------------------------------------ seeding (modes 3, 4)
@@ -1381,18 +1404,27 @@ constexpr int STEP_MIN_BLOCKS_PAPER = 4;
 // registers per thread) spill less.
 constexpr int STEP_MIN_BLOCKS_COOP = 4;
 
-// The mixed kernels (modes 2, 3) are bound by latency rather than a pipe (instruction
-// fetch, dependent df64 chains), and more resident warps hide more of it than the extra
-// spills cost: 12 blocks per SM (40 registers per thread).  Measured on the 128^3 slab,
-// mixed / seeded mixed ms: 8 blocks 67.1 / 56.6, 10: 58.6 / 52.6, 12: 58.1 / 51.0,
-// 16: 57.9 / 52.7.
-constexpr int STEP_MIN_BLOCKS_MIXED = 12;
+// The mixed kernels (modes 2, 3) are bound by instruction fetch: their code exceeds the
+// instruction caches, and warps at unrelated places of it stream it one by one.  A large
+// block that meets at the start of each substep, after its start sources and before its
+// polish (block_meet) runs one part of the code at a time.  128^3 slab seeded / 300k stiff
+// cells mixed, ms: no meeting, 12 blocks of 128 (40 registers) 51.5 / 20.0; with lanes that
+// meet again after every branch of the substep 49.8 / 12.6; the block meeting three times
+// 46.7 / 11.4; 8 blocks of 128 (64 registers) 44.4 / 11.3; 4 blocks of 256 36.2 / 9.7; 2 of
+// 512 33.5 / 9.0; 3 of 512 (40 registers) 35.2 / 9.3; 1 of 768 35.3 / 9.8; 1 of 1024 34.6 / 10.2.
+constexpr int STEP_THREADS = 128;
+constexpr int STEP_THREADS_MIXED = 512;
+constexpr int STEP_MIN_BLOCKS_MIXED = 2;
+constexpr int step_threads(int mode, int lpc) {
+  return (lpc == 1 && (mode == 2 || mode == 3)) ? STEP_THREADS_MIXED : STEP_THREADS;
+}
 
 template <int MODE, bool BATCH, int LPC = 1>
-__global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? STEP_MIN_BLOCKS_MIXED
-                                                      : (MODE == 0) ? STEP_MIN_BLOCKS_PAPER
-                                                                    : STEP_MIN_BLOCKS)
-                                                  : STEP_MIN_BLOCKS_COOP)
+__global__ void __launch_bounds__(step_threads(MODE, LPC),
+                                  (LPC == 1) ? ((MODE == 2 || MODE == 3) ? STEP_MIN_BLOCKS_MIXED
+                                                : (MODE == 0)            ? STEP_MIN_BLOCKS_PAPER
+                                                                         : STEP_MIN_BLOCKS)
+                                             : STEP_MIN_BLOCKS_COOP)
     k_step(DevFields f1, const BoxTable* __restrict__ boxes, DevParams p, double dt, unsigned long long* cursor,
            long long ntotal, const MlpDev* __restrict__ mlp) {
   static_assert(LPC == 1 || ((MODE == 1 || MODE == 2) && !BATCH), "cooperative kernels: modes 1 and 2, one box");
@@ -1410,7 +1442,8 @@ __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? 
   DevFields fb;
   long long li = -1;   // local cell index within its box
   bool have = false;
-  bool done = false;   // the work queue is empty for this lane
+  // the work queue is empty for this lane, or the lane's group of a sparse warp takes no cells
+  bool done = LPC > 1 && (int)((threadIdx.x & 31u) / LPC) >= p.groups;
   while (true) {
     if (!have && !done) {
       long long gi = claim_cells_lpc<LPC>(cursor);
@@ -1478,8 +1511,8 @@ __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? 
     }
     if constexpr (SEEDED) {
       // The seed network runs on the warp's tensor cores, an instruction all 32 lanes
-      // issue together: lanes stay in the loop until the whole warp is done.
-      if (__all_sync(0xffffffffu, done)) break;
+      // issue together, and the block runs in step: threads stay until it is done.
+      if (__syncthreads_and(done)) break;
       bool need = false, last = false;
       double dts = 0.0, src[3] = {0.0, 0.0, 0.0}, g[3];
       if (have && s.t < dt) {
@@ -1496,34 +1529,41 @@ __global__ void __launch_bounds__(128, (LPC == 1) ? ((MODE == 2 || MODE == 3) ? 
       seed_features(lf, c, s, dts, src, need, g, feat);
       __syncwarp();
       mlp_infer_warp(p.mlp_mma, feat, o);
-      if (need) {
-        double seed[3];
-        const bool ok = seed_from_outputs(o, g, s, p, seed);
-        if constexpr (MODE == 3)
-          substep_mixed_solve(c, cd, cf, p, dt, dts, last, s, xe_gf, td_gf, td_hp, ok ? seed : nullptr);
-        else solve_substep64(c, p, dt, dts, last, s, xe_g, td_g, ok ? seed : nullptr, &cf);
-        if (!finite3(s.Tmu, s.xH2, s.xHp)) {
-          s.status |= ST_NONFIN;
-          s.t = dt;
-        }
+      double seed[3];
+      const bool ok = need && seed_from_outputs(o, g, s, p, seed);
+      block_meet<true>();
+      if constexpr (MODE == 3) {
+        substep_mixed_solve<1, true>(c, cd, cf, p, dt, dts, last, s, xe_gf, td_gf, td_hp, ok ? seed : nullptr, need);
+      } else {
+        if (need) solve_substep64(c, p, dt, dts, last, s, xe_g, td_g, ok ? seed : nullptr, &cf);
+      }
+      if (need && !finite3(s.Tmu, s.xH2, s.xHp)) {
+        s.status |= ST_NONFIN;
+        s.t = dt;
       }
     } else {
-      if (done) break;
-      if (s.t < dt) {
-        if (s.nsub >= p.max_sub) {
-          s.status |= ST_MAX_SUB;
-          s.t = dt;
-        } else if constexpr (MODE == 0) {
-          substep_paper(c, p, dt, s);
-        } else if constexpr (MODE == 1) {
-          substep_newton64<LPC>(c, cf, p, dt, s, xe_g, td_g);
-        } else if constexpr (MODE == 2) {
-          substep_mixed<LPC>(c, cd, cf, p, dt, s, xe_gf, td_gf, td_hp);
-        }
-        if (!finite3(s.Tmu, s.xH2, s.xHp)) {
-          s.status |= ST_NONFIN;
-          s.t = dt;
-        }
+      // modes 1 and 2 with one lane per cell: threads stay until their block is done
+      constexpr bool SYNC = (MODE == 1 || MODE == 2) && LPC == 1;
+      if constexpr (SYNC) {
+        if (__syncthreads_and(done)) break;
+      } else {
+        if (done) break;
+      }
+      bool need = have && s.t < dt;
+      if (need && s.nsub >= p.max_sub) {
+        s.status |= ST_MAX_SUB;
+        s.t = dt;
+        need = false;
+      }
+      if constexpr (MODE == 2) {
+        substep_mixed<LPC, SYNC>(c, cd, cf, p, dt, s, xe_gf, td_gf, td_hp, need);
+      } else if (need) {
+        if constexpr (MODE == 0) substep_paper(c, p, dt, s);
+        else substep_newton64<LPC>(c, cf, p, dt, s, xe_g, td_g);
+      }
+      if (need && !finite3(s.Tmu, s.xH2, s.xHp)) {
+        s.status |= ST_NONFIN;
+        s.t = dt;
       }
     }
     if (have && !(s.t < dt)) {

@@ -141,6 +141,7 @@ struct DevParams {
   int newton_max, max_sub;
   unsigned flags;
   const unsigned* order = nullptr;  // optional: the k-th claimed cell is order[k] (cost-ordered queue)
+  int groups = 8;  // cooperative kernels: cells a warp advances at once (of 32 / lanes per cell)
   const MlpMma* mlp_mma = nullptr;  // seeded modes: the network for the warp-level inference
 };
 
