@@ -560,8 +560,8 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 // with its damping, predictor and halving decisions.  (Damping here too solved some substeps
 // that the plain iteration halves, which changed the substep grid of 5 in 13,824 cells near
 // x_H = 0.)
-constexpr int TAN_MAXIT = 12;
-constexpr int TAN_MAXIT32 = 8;
+constexpr int TAN_MAXIT = 16;
+constexpr int TAN_MAXIT32 = 16;
 constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
 
 // source_tangents over the cell's lanes: with four, each takes one direction (the last
@@ -633,16 +633,25 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
         }
       }
       ok = solve3<float>(J, r, u);
+      // damped as in damped_step, but for its x_H bound: where that would act, the plain
+      // iteration's own decisions count
+      bool whole = true;
+      float lamT = (u[0] < -0.99f) ? -0.99f / u[0] : 1.0f, lamX = 1.0f;
+#pragma unroll
+      for (int i = 1; i < 3; ++i)
+        if (u[i] < -1e-8f) lamX = fminf(lamX, -0.99f * x[i] / u[i]);
+      ok = ok && lamX * (-2.0f * u[1] - u[2]) >= -0.98f * xH;
+      whole = lamT >= 1.0f && lamX >= 1.0f;
+      u[0] *= lamT;
       float rel = fabsf(u[0]);
 #pragma unroll
       for (int i = 1; i < 3; ++i) {
-        if (!(u[i] >= -0.98f * x[i])) {
-          ok = ok && fabsf(u[i]) <= 1e-8f;
-          u[i] = -0.98f * x[i];  // too little to matter to the others; phase 2 settles it
-        }
+        const bool tiny = fabsf(u[i]) <= 1e-8f;
+        u[i] *= lamX;
+        if (tiny && u[i] < -0.99f * x[i]) u[i] = -0.99f * x[i];  // phase 2 settles it
         rel = fmaxf(rel, fabsf(u[i]) / (x[i] + u[i] + 1e-8f));
       }
-      ok = ok && u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * xH && isfinite(rel);
+      ok = ok && isfinite(rel);
       if (!ok) break;
       D[0] += a * u[0];
       D[1] += u[1];
@@ -651,14 +660,14 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       td = v.td + v.dtd[0] * u[0] + v.dtd[1] * u[1] + v.dtd[2] * u[2];
 #pragma unroll
       for (int i = 0; i < 3; ++i) dtd[i] = v.dtd[i];
-      if (rel < 3e-5f) break;
-      if (it32 > 2 && !(rel <= 0.5f * prev)) {
+      if (whole && rel < 3e-5f) break;
+      if (whole && !(rel <= 0.5f * prev) && it32 > 2) {
         ok = rel < 1e-3f;  // FP32's rounding floor
         break;
       }
       ok = it32 < TAN_MAXIT32;
       if (!ok) break;
-      prev = rel;
+      prev = whole ? rel : 3e38f;
     }
     y[0] = yn[0] + yn[0] * double(D[0]);
 #pragma unroll
@@ -758,7 +767,9 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       res = it32 + it;
       break;
     }
-    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev)) break;
+    // not contracting; steps below 1e-4 go on (in hot gas the rounding of x_H = 1 - 2 x_H2 -
+    // x_H+ moves x_H2 by that much until an iterate repeats)
+    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev) && rel > 1e-4f) break;
     fresh = prev > 0.0f && rel > 1e-3f * prev;
     prev = rel;
     // the next evaluation's inner roots, predicted along the step
