@@ -560,7 +560,7 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 // with its damping, predictor and halving decisions.  (Damping here too solved some substeps
 // that the plain iteration halves, which changed the substep grid of 5 in 13,824 cells near
 // x_H = 0.)
-constexpr int TAN_MAXIT = 16;
+constexpr int TAN_MAXIT = 12;
 constexpr int TAN_MAXIT32 = 16;
 constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
 
@@ -711,6 +711,10 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
         J[i][0] = J[i][3 - i] = 0.0f;
       }
     }
+    // what one rounding of the other unknowns moves an abundance by
+    const float eps = 1.2e-16f;
+    const float noise[3] = {0.0f, eps * (fabsf(J[1][0]) + fabsf(J[1][2]) * xp) / fabsf(J[1][1]),
+                            eps * (fabsf(J[2][0]) + fabsf(J[2][1]) * x2) / fabsf(J[2][2])};
     ok = solve3<float>(J, r, u);
     // T_mu, x_H2, x_H+ and x_H must keep 2% of their values (damped_step limits at 1%),
     // except an abundance whose step is below 1e-8 (too little to matter to the others): it
@@ -734,7 +738,9 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       }
       const double yi = y[i] + d[i];
       const float ri = trace ? float(fabs(d[i]) / (fabs(yi) + 1e-300)) : fabsf(u[i]) / (fabsf(float(yi)) + 1e-30f);
-      rel = fmaxf(rel, ri);
+      // (in hot gas the rounding of x_H = 1 - 2 x_H2 - x_H+ moves x_H2 by up to 1e-5 of itself,
+      // back and forth: such a step is no distance from the root)
+      if (!(fabsf(u[i]) <= noise[i])) rel = fmaxf(rel, ri);
     }
     ok = ok && u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * float(xH) && isfinite(rel);
     if (!ok) break;
@@ -767,9 +773,7 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       res = it32 + it;
       break;
     }
-    // not contracting; steps below 1e-4 go on (in hot gas the rounding of x_H = 1 - 2 x_H2 -
-    // x_H+ moves x_H2 by that much until an iterate repeats)
-    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev) && rel > 1e-4f) break;
+    if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev)) break;
     fresh = prev > 0.0f && rel > 1e-3f * prev;
     prev = rel;
     // the next evaluation's inner roots, predicted along the step
