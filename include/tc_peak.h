@@ -8,7 +8,7 @@
  * events on the same stream).  Operations per launch = grid * block * chains * iters.
  *   kind 0: FP64 fused multiply-add      kind 1: FP32 fused multiply-add
  *   kind 2: FP64 exp (the step's, tc_exp64.cuh)  kind 3: FP64 log (the same)
- *   kind 4: FP64 sqrt()                  kind 5: FP64 division
+ *   kind 4: FP64 sqrt()                  kind 5: FP64 division (the step's)
  *   kind 6: FP64 pow(x, y)               kind 7: FP32 expf()
  *   kind 8: FP32 __expf(), the approximate exponential of the fast-math mixed kernels:
  *           one MUFU ex2 per operation, so its rate is the MUFU pipe's

@@ -5,7 +5,7 @@
 
 #include "../../include/tc.h"
 #include "../../include/tc_peak.h"
-#include "tc_exp64.cuh"
+#include "tc_phys.cuh"
 
 namespace tcg {
 int df64_peak_launch(int kind, int grid, int block, int iters, double* sink, void* stream);  // tc_df64_diag.cu
@@ -42,7 +42,7 @@ __global__ void k_peak(int iters, double* sink) {
         if (KIND == 2) v[c] = tcg::exp64(-v[c]);          // converges to the omega constant
         if (KIND == 3) v[c] = tcg::log64(v[c] + 2.0);      // converges to ~1.146
         if (KIND == 4) v[c] = sqrt(v[c] + 1.0);     // converges to the golden ratio
-        if (KIND == 5) v[c] = 1.0 / (v[c] + 1.0);   // converges to 0.618
+        if (KIND == 5) v[c] = tcg::m_div(1.0, v[c] + 1.0);   // converges to 0.618
         if (KIND == 6) v[c] = pow(v[c] + 1.0, 0.7);
       }
     }
