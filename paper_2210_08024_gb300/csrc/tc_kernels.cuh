@@ -190,7 +190,7 @@ TCG_FN void substep_paper(const CellC<double>& c, const DevParams& p, double dt,
       Tev = s.mu * (s.Tmu + p.fd_rel * s.Tmu);
       Tdf = Td0;
     }
-    ChemT<double> b = chem_T(c, Tev, p.flags);
+    ChemT<double> b = chem_T(c, Tev, p.flags, false);
     CoolT<double> k = cool_T(c, b, p.flags);
     Equil<double> q;
     q.xe = s.xe; q.xCp = s.xCp; q.xCO = s.xCO;
@@ -520,7 +520,7 @@ template <class F>
 TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneState& s, F& td_g, double& H0,
                           double& CH2, double& CHp) {
   const double T = s.mu * s.Tmu;
-  ChemT<F> b = chem_T(cf, to_prec<F>(T), p.flags);
+  ChemT<F> b = chem_T(cf, to_prec<F>(T), p.flags, false);
   CoolT<F> k = cool_T(cf, b, p.flags);
   Equil<F> q;
   q.xe = to_prec<F>(s.xe); q.xCp = to_prec<F>(s.xCp); q.xCO = to_prec<F>(s.xCO);
