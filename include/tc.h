@@ -177,10 +177,11 @@ typedef struct tc_tune_choice {
 } tc_tune_choice;
 
 /* Autotuner of the step launch.  Times one step of the cells of *f (device pointers, as
- * for tc_step) in every candidate shape -- 32, 64 or 128 threads per block (256 or 512 too for
- * the mixed modes on launches that fill the GPU), the occupancy limit or 4 resident blocks per SM, and for modes TC_MODE_NEWTON_FP64 and TC_MODE_MIXED
- * one or four lanes per cell (four only when the cooperative kernel holds the cells in
- * at most 8 waves of its resident lanes) -- with CUDA events on `stream`, each candidate
+ * for tc_step) in every candidate shape -- the default shape of the launch's size, and 32, 64 or
+ * 128 threads per block (256 or 512 too for the mixed modes on launches that fill the GPU),
+ * the occupancy limit or 4 resident blocks per SM, and for modes TC_MODE_NEWTON_FP64 and
+ * TC_MODE_MIXED one or four lanes per cell (four only when the cooperative kernel holds the
+ * cells in at most 8 waves of its resident lanes) -- with CUDA events on `stream`, each candidate
  * once, or three times (fastest kept) when one step takes under 20 ms, and records the fastest
  * for the size class floor(log2(ncell)) in the handle: later tc_step and tc_step_host
  * calls of that size class whose tc_params leave block, blocks_per_sm and

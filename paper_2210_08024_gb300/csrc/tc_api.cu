@@ -266,22 +266,41 @@ static int coop_occupancy(int kmode, int block) {
 // class; otherwise the rules below and the occupancy limit.  The persistent grid never
 // exceeds the blocks that hold every cell at once.
 struct Shape {
-  int grid, block, lpc, groups;
+  int grid, block, lpc, groups, per_sm;  // per_sm: 0 = the occupancy limit
 };
-// Threads per block where neither the caller nor the autotuner chose.  Launches of few cells
-// take blocks of one warp: they spread over the SMs, and no lane waits for a block's other
-// warps (random states by FP64 Newton, one lane per cell, 32 / 128 threads: 4096 cells 49 / 61
-// ms, 8000 46 / 58; 12,800 curve cells 15.1 / 15.7).  The mixed kernels' large blocks run in
-// step and fetch their code once (tc_kernels.cuh), which pays as soon as the cells fill them.
-// ms at 32 / 128 / 256 / 512 threads: seeded mixed, slab cells: 20k 5.4 / 5.5 / 5.8 / 6.4, 60k
-// 6.8 / 6.4 / 6.6 / 6.6, 150k 10.3 / 9.3 / 8.3 / 9.2, 300k 14.8 / 11.8 / 10.5 / 10.5, 2M 44.4
-// (128) / 36.2 / 33.5; random states: 4k 40 / 44 / 50 / 62, 30k 76 / 58 / 59 / 69, 100k 178 /
-// 155 / 114 / 98.
-static int default_block(int kmode, long long ntotal, int num_sms) {
+// Threads per block and resident blocks per SM (0: the occupancy limit) where neither the
+// caller nor the autotuner chose, one lane per cell, by the cells per SM.
+//  - Few cells take blocks of one warp: they spread over the SMs, and no lane waits for a
+//    block's other warps (random states by FP64 Newton, 32 / 128 threads: 4096 cells 49 / 61
+//    ms, 8000 46 / 58; 12,800 curve cells 15.1 / 15.7).
+//  - FP64 modes: one warp per SM partition nearly fills its FP64 pipe (65 cycles an
+//    instruction, 77 with more), and fewer lanes take more cells each, longest first, so that
+//    lanes finish together.  More warps pay, by covering the rest, when each lane still gets
+//    a dozen cells.  ms at 4 / 8 / 16 warps per SM / the limit: slab by FP64 Newton 100k 7.0 /
+//    8.3 / 8.2 / 8.0, 300k 9.2 / 9.8 / 12.6 / 14.5, 600k 18.9 / 15.3 / 18.7 / 22.0, 1M 31.9 / 26.0
+//    / 26.1 / 30.2, 2M 67.6 / 55.0 / 55.3 / 51.7; by the paper's scheme 100k 3.0 / 4.2 / 5.4 / 5.5,
+//    300k 5.8 / 5.9 / 8.8 / 8.7, 885k 13.6 / 12.0 / 11.7 / 11.7; random states by FP64 Newton 30k
+//    58 / 67 / 72 / 66, 100k 113 / 97 / 128 / 147; seeded FP64 300k 33 / 43 / 54 / 57.
+//  - Mixed modes: large blocks run in step and fetch their code once (tc_kernels.cuh), which
+//    pays as soon as the cells fill them.  ms at 32 / 128 / 256 / 512 threads: seeded mixed, slab
+//    cells: 20k 5.4 / 5.5 / 5.8 / 6.4, 60k 6.8 / 6.4 / 6.6 / 6.6, 150k 10.3 / 9.3 / 8.3 / 9.2, 300k
+//    14.8 / 11.8 / 10.5 / 10.5, 2M 44.4 (128) / 36.2 / 33.5; random states: 4k 40 / 44 / 50 / 62, 30k
+//    76 / 58 / 59 / 69, 100k 178 / 155 / 114 / 98.  At 100k one block of 256 an SM instead of
+//    the limit: slab seeded 7.2 -> 6.7, random states mixed 74 -> 62.
+static void default_block(int kmode, long long ntotal, int num_sms, int& b, int& per_sm) {
   const long long per = ntotal / num_sms;
-  if (per < 112) return 32;
-  if (kmode != 2 && kmode != 3) return tcg::STEP_THREADS;
-  return (per < 600) ? 128 : (per < 1600) ? 256 : 512;
+  per_sm = 0;
+  if (per < 112) {
+    b = 32;
+  } else if (kmode == 2 || kmode == 3) {
+    b = (per < 600) ? 128 : (per < 1600) ? 256 : 512;
+    if (b == 256 && per < 1200) per_sm = 1;
+  } else {
+    b = (per < 1200) ? 64 : 128;
+    if (per < 1200) per_sm = 2;
+    else if (per < 2600) per_sm = 1;
+    else if (per < ((kmode == 0) ? 5000 : 9000)) per_sm = 2;
+  }
 }
 
 // Whether a launch of modes 1 and 2 takes four lanes per cell: while the cells' warps of
@@ -319,8 +338,18 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
   if (!coop_ok) lpc = 1;
   if (lpc <= 0) lpc = (coop_ok && default_coop(kmode, ntotal, h->num_sms)) ? 4 : 1;
   if (lpc != 4) lpc = 1;
-  if (auto_block) b = default_block(kmode, ntotal, h->num_sms);
-  if (lpc == 4 && b > tcg::STEP_THREADS) b = tcg::STEP_THREADS;
+  if (auto_block) {
+    int ps = 0;
+    default_block(kmode, ntotal, h->num_sms, b, ps);
+    if (lpc == 4) {
+      if (b > tcg::STEP_THREADS) b = tcg::STEP_THREADS;
+    } else if (per_sm <= 0) {
+      per_sm = ps;
+    }
+  } else if (lpc == 4 && b > tcg::STEP_THREADS) {
+    b = tcg::STEP_THREADS;
+  }
+  const int chosen = per_sm > 0 ? per_sm : 0;
   if (per_sm <= 0) {
     per_sm = (lpc == 4) ? coop_occupancy(kmode, b)
              : (kmode == 0) ? tcg::occupancy_mode0_impl(b)
@@ -333,7 +362,7 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
   long long need = ((ntotal + groups - 1) / groups * 32 + b - 1) / b;
   if (g > need) g = need;
   if (g < 1) g = 1;
-  return Shape{(int)g, b, lpc, groups};
+  return Shape{(int)g, b, lpc, groups, chosen};
 }
 
 // Grows the cost-ordering workspace to ncell cells (not while `st` is being captured).
@@ -475,21 +504,24 @@ int tc_autotune(tc_handle* h, const tc_fields* f, double dt_s, void* stream, tc_
   h->p.lanes_per_cell = 0;
   rc = run(&ms0);
   const int reps = (rc == TC_OK && ms0 < 20.f) ? 3 : 1;
+  const Shape def = launch_shape(h, kmode, false, f->ncell);
   tc_tune_choice bestc = {0, 0, 0, 3.4e38f};
+  auto candidate = [&](int block, int per_sm, int lpc) {
+    h->p.block = block;
+    h->p.blocks_per_sm = per_sm;
+    h->p.lanes_per_cell = lpc;
+    float tmin = 3.4e38f;
+    for (int r = 0; r < reps && rc == TC_OK; ++r) {
+      float ms = 0.f;
+      rc = run(&ms);
+      if (ms < tmin) tmin = ms;
+    }
+    if (rc == TC_OK && tmin < bestc.ms) bestc = tc_tune_choice{block, per_sm, lpc, tmin};
+  };
+  candidate(def.block, def.per_sm, def.lpc);
   for (int ib = 0; ib < nblk && rc == TC_OK; ++ib)
     for (int ip = 0; ip < 2 && rc == TC_OK; ++ip)
-      for (int il = 0; il < (coop_ok ? 2 : 1) && rc == TC_OK; ++il) {
-        h->p.block = blocks[ib];
-        h->p.blocks_per_sm = per_sms[ip];
-        h->p.lanes_per_cell = lpcs[il];
-        float tmin = 3.4e38f;
-        for (int r = 0; r < reps && rc == TC_OK; ++r) {
-          float ms = 0.f;
-          rc = run(&ms);
-          if (ms < tmin) tmin = ms;
-        }
-        if (rc == TC_OK && tmin < bestc.ms) bestc = tc_tune_choice{blocks[ib], per_sms[ip], lpcs[il], tmin};
-      }
+      for (int il = 0; il < (coop_ok ? 2 : 1) && rc == TC_OK; ++il) candidate(blocks[ib], per_sms[ip], lpcs[il]);
   h->p = saved;
   if (rc == TC_OK) {
     h->tuned[size_class(f->ncell)] = tc_handle::Tuned{1, bestc.block, bestc.blocks_per_sm, bestc.lanes_per_cell};

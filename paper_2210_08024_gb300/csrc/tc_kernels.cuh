@@ -1303,15 +1303,18 @@ TCG_FN void substep_mixed_solve(const CellC<double>& c, const CellC<df64>& cd, c
     } while (again);
   }
   block_meet<SYNC>();
-  if (!need) return;
   Equil<df64> qlast;
   const int it32 = it;
   bool have32 = false;
   double y32[3];
-  if (it >= 0) {
+  if (need && it >= 0) {
     y32[0] = y[0]; y32[1] = y[1]; y32[2] = y[2];
     have32 = true;
     fd_jacobian32<LPC>(cf, p, s.mu, Kinv, dts, y, xe_g, td_g, J);
+  }
+  block_meet<SYNC>();
+  if (!need) return;
+  if (it >= 0) {
     df64 xg = df64::make(xe_g, 0.0f), tg = df64::make(td_g, 0.0f);
     if (!polish_hp<df64>(cd, p, s.mu, Kinv, yn, dts, y, J, xg, tg, qlast)) it = -1;
   }
@@ -1421,12 +1424,13 @@ constexpr int STEP_MIN_BLOCKS_COOP = 4;
 
 // The mixed kernels (modes 2, 3) are bound by instruction fetch: their code exceeds the
 // instruction caches, and warps at unrelated places of it stream it one by one.  A large
-// block that meets at the start of each substep, after its start sources and before its
-// polish (block_meet) runs one part of the code at a time.  128^3 slab seeded / 300k stiff
-// cells mixed, ms: no meeting, 12 blocks of 128 (40 registers) 51.5 / 20.0; with lanes that
-// meet again after every branch of the substep 49.8 / 12.6; the block meeting three times
-// 46.7 / 11.4; 8 blocks of 128 (64 registers) 44.4 / 11.3; 4 blocks of 256 36.2 / 9.7; 2 of
-// 512 33.5 / 9.0; 3 of 512 (40 registers) 35.2 / 9.3; 1 of 768 35.3 / 9.8; 1 of 1024 34.6 / 10.2.
+// block that meets at the start of each substep, after its start sources, and before and
+// after the FP32 Jacobian at the root (block_meet) runs one part of the code at a time.  128^3
+// slab seeded / 300k stiff cells mixed, ms: no meeting, 12 blocks of 128 (40 registers) 51.5 /
+// 20.0; with lanes that meet again after every branch of the substep 49.8 / 12.6; the block
+// meeting three times 46.7 / 11.4; 8 blocks of 128 (64 registers) 44.4 / 11.3; 4 blocks of 256
+// 36.2 / 9.7; 2 of 512 33.5 / 9.0; 3 of 512 (40 registers) 35.2 / 9.3; 1 of 768 35.3 / 9.8; 1 of
+// 1024 34.6 / 10.2; 2 of 512 meeting four times 32.9 / 8.9.
 constexpr int STEP_THREADS = 128;
 constexpr int STEP_THREADS_MIXED = 512;
 constexpr int STEP_MIN_BLOCKS_MIXED = 2;

@@ -103,8 +103,7 @@ TCG_FN float m_abs(float a) { return fabsf(a); }
 // Quotients of the FP64 physics on the device: the approximate reciprocal (MUFU, ~2^-20), one
 // third-order step and one residual correction, 6 FP64 instructions and no slow path; error
 // below 0.51 ulp (tests/test_gpu_div64.py).  Exponents from which a step could leave the range
-// take the plain division.  Other types (and the mixed kernels' rare FP64) divide.
-template <class A, class B> TCG_FN auto m_div(A a, B b) -> decltype(a / b) { return a / b; }
+// take the plain division.
 TCG_FN double m_div(double a, double b) {
 #if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_EXP64)
   if ((unsigned)((hi_word(b) & 0x7fffffff) - 0x10000000) < 0x60000000u &&
@@ -119,6 +118,18 @@ TCG_FN double m_div(double a, double b) {
 #endif
   return a / b;
 }
+
+// A divisor, `a / over(b)`: plain for every type but the device's FP64, which divides by m_div.
+// (A function of both operands instead changed how the compiler forms the mixed kernels' FP32
+// expressions, and with it their last bits.)
+struct OverF64 {
+  double b;
+};
+TCG_FN double operator/(double a, OverF64 d) { return m_div(a, d.b); }
+template <class F> TCG_FN F over(F b) { return b; }
+#if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_EXP64)
+TCG_FN OverF64 over(double b) { return OverF64{b}; }
+#endif
 
 // Precision traits of the scalar types: the relative tolerance of the inner root solves
 // (C/O/e equilibrium, dust temperature), a little above each type's rounding; whether
@@ -150,7 +161,7 @@ template <class F> struct ConstOf { using type = F; };
 template <class F> TCG_FN F to_prec(double x) { return F(x); }
 template <> TCG_FN df64 to_prec<df64>(double x) { return to_df64(x); }
 
-template <class F> TCG_FN F logistic(F z) { return m_div(F(1), F(1) + m_exp(-z)); }
+template <class F> TCG_FN F logistic(F z) { return F(1) / over(F(1) + m_exp(-z)); }
 
 // Parameters copied to the device by value with each launch.
 struct MlpMma;  // seed network in the tensor-core layout (tc_mlp_mma.cuh)
@@ -291,7 +302,7 @@ template <class F, class FC> TCG_FN F xe_hot_of(const CellC<FC>& c, F lt) {
   F xeHe;
   if constexpr (Prec<F>::cls == 0) {  // one quotient (the product stays below 1e70)
     F a = K(1) + eHe, b = K(1) + eHe * K(4160.262005375057);
-    xeHe = m_div(K(0.1) * (a + b), a * b);
+    xeHe = K(0.1) * (a + b) / over(a * b);
   } else {
     xeHe = K(0.1) * (K(1) / (K(1) + eHe) + K(1) / (K(1) + eHe * K(4160.262005375057)));  // exp(25/3)
   }
@@ -309,19 +320,19 @@ template <class F, class FC> TCG_BIG ChemT<F> chem_T(const CellC<FC>& c, F T, un
   b.T = T;
   b.lnT = m_log(T);
   b.sqT = m_sqrt(T);
-  const F invT = m_div(K(1), T);
+  const F invT = K(1) / over(T);
   b.invT = invT;
-  b.S = m_div(K(1), K(1) + m_exp(K(-10.0 / 1.5e4) * (T - K(2.75e4))));
+  b.S = K(1) / over(K(1) + m_exp(K(-10.0 / 1.5e4) * (T - K(2.75e4))));
   if (flags & FL_CONST_KGR) {
     b.kgr = K(3.0e-17) * c.Zd;
   } else {
     F s2 = b.sqT * K(0.1);  // sqrt(T/100)
     F T2 = T * K(0.01);
-    b.kgr = m_div(K(3.0e-17) * c.Zd * K(2) * s2, K(1) + K(0.4) * s2 + K(0.2) * T2 + K(0.08) * T2 * T2);
+    b.kgr = K(3.0e-17) * c.Zd * K(2) * s2 / over(K(1) + K(0.4) * s2 + K(0.2) * T2 + K(0.08) * T2 * T2);
   }
   F lT4 = b.lnT - K(9.210340371976184);  // ln(T/1e4)
   b.arr = K(2.54e-13) * m_exp((K(-0.8163) - K(0.0208) * lT4) * lT4);
-  b.kci = m_div(K(5.85e-11) * b.sqT * m_exp(K(-157809.1) * invT), K(1) + b.sqT * K(0.003162277660168379));
+  b.kci = K(5.85e-11) * b.sqT * m_exp(K(-157809.1) * invT) / over(K(1) + b.sqT * K(0.003162277660168379));
   b.kcdH = K(6.67e-12) * b.sqT * m_exp(K(-1) - K(63593.0) * invT);
   b.kcdH2 = K(5.996e-30) * m_exp(K(4.1881) * b.lnT - K(54657.4) * invT - K(5.6881) * m_log(K(1) + K(6.761e-6) * T));
   b.wdH3T = K(WDH3) * m_exp(K(WDH4) * b.lnT);
@@ -361,8 +372,8 @@ template <class F> struct CoolT {
 // E_21/k_B = 1.184e5 K, from ln(T/1e4) and 1e4/T.
 template <class F> TCG_FN F lya_of(F lT4, F invT4) {
   using K = typename ConstOf<F>::type;
-  return m_div(K(1.184e5 * KB * 5.31e-8) * m_exp(K(0.15) * lT4 - K(11.84) * invT4),
-               K(1) + m_exp(K(0.65) * (lT4 - K(1.6094379124341003))));
+  return K(1.184e5 * KB * 5.31e-8) * m_exp(K(0.15) * lT4 - K(11.84) * invT4) /
+         over(K(1) + m_exp(K(0.65) * (lT4 - K(1.6094379124341003))));
 }
 // free-free Gaunt factor at log10 T = lt
 template <class F> TCG_FN F gff_of(F lt) {
@@ -375,7 +386,7 @@ template <class F> TCG_FN F gff_of(F lt) {
 template <class F> TCG_FN F rovib_lte_of(F lT3, F iT3) {
   using K = typename ConstOf<F>::type;
   F q = K(0.13) * iT3;
-  F Lrot = m_div(K(9.5e-22) * m_exp(K(3.76) * lT3 - q * q * q), K(1) + K(0.12) * m_exp(K(2.1) * lT3)) +
+  F Lrot = K(9.5e-22) * m_exp(K(3.76) * lT3 - q * q * q) / over(K(1) + K(0.12) * m_exp(K(2.1) * lT3)) +
            K(3e-24) * m_exp(K(-0.51) * iT3);
   F Lvib = K(6.7e-19) * m_exp(K(-5.86) * iT3) + K(1.6e-18) * m_exp(K(-11.7) * iT3);
   return Lrot + Lvib;
@@ -395,7 +406,7 @@ template <class F, class FC> TCG_BIG CoolT<F> cool_T(const CellC<FC>& c, const C
   const F T = b.T, lnT = b.lnT;
   const F invT = b.invT;
   k.fcA = K(1.0e-12) * b.sqT * m_exp(K(-1000.0) * invT);
-  k.fcB = K(1.4e-12) * b.sqT * m_exp(m_div(K(-18100.0), T + K(1200.0)));
+  k.fcB = K(1.4e-12) * b.sqT * m_exp(K(-18100.0) / over(T + K(1200.0)));
   k.eps_num = K(5.22) + K(2.25) * m_exp(K(0.147) * lnT);
   F lT4 = lnT - K(9.210340371976184);
   F invT4 = K(1e4) * invT;
@@ -576,20 +587,20 @@ template <class F> TCG_BIG Equil<F> equilibrium(const CellC<F>& c, const ChemT<F
   // x_C+(x), its derivative, ln psi(x) and d ln psi / dx
   auto xcp = [&](F x, F& dxcp, F& lp, F& dlp) -> F {
     F ne = x * c.n;
-    F psi = m_div(Gs, m_max(ne, F(1e-30))) + F(50);
+    F psi = Gs / over(m_max(ne, F(1e-30))) + F(50);
     lp = m_log(psi);
     F pa = m_exp(F(WDC2) * lp);
     F pb = b.wdC3T * m_exp(b.wdCex * lp);
     F D = F(1) + F(WDC1) * pa * (F(1) + pb);
-    F invD = m_div(F(1), D);
+    F invD = F(1) / over(D);
     F agr = agr0 * invD;
     F den = sink0 + (agr + b.arrC * x) * c.n;
     // dD/dx = dD/d ln psi  d ln psi/dx, with dD/d ln psi = C1 (C2 pa (1 + pb) + pa C5' pb)
     // and d ln psi/dx = -(psi - 50)/(psi x) when ne > floor; d agr/dx = -agr dD/dx / D
-    dlp = (ne > F(1e-30)) ? m_div(-(psi - F(50)), psi * x) : F(0);
+    dlp = (ne > F(1e-30)) ? -(psi - F(50)) / over(psi * x) : F(0);
     F dDdx = F(WDC1) * (F(WDC2) * pa * (F(1) + pb) + pa * b.wdCex * pb) * dlp;
     F dagr = -agr * invD * dDdx;
-    F invden = m_div(F(1), den);
+    F invden = F(1) / over(den);
     F r = num * invden;
     dxcp = -r * invden * ((dagr + b.arrC) * c.n);
     return r;
@@ -615,7 +626,7 @@ template <class F> TCG_BIG Equil<F> equilibrium(const CellC<F>& c, const ChemT<F
       if (g == F(0)) { xe = x; break; }
       if (g > F(0)) hi = x; else lo = x;
       F gp = F(1) - w * d;
-      F xn = x - m_div(g, gp);
+      F xn = x - g / over(gp);
       // a Newton step that lands on a bracket end is kept: near the root the bracket
       // collapses onto it, and bisecting there would only grind the bracket down
       const bool newton = (xn >= lo && xn <= hi);
@@ -648,8 +659,8 @@ template <class F> TCG_BIG Equil<F> equilibrium(const CellC<F>& c, const ChemT<F
     F dd, dl;
     q.xCp = xcp(xe, dd, q.lpsi, dl);
   }
-  F fr = m_max((c.xCtot > F(0)) ? m_div(q.xCp, c.xCtot) : F(0), xHp);
-  q.xCO = m_div(c.xCtot * F(2) * xH2 * (F(1) - fr), F(1) + c.rCO2);  // Eq. e:CO
+  F fr = m_max((c.xCtot > F(0)) ? q.xCp / over(c.xCtot) : F(0), xHp);
+  q.xCO = c.xCtot * F(2) * xH2 * (F(1) - fr) / over(F(1) + c.rCO2);  // Eq. e:CO
   q.xC = c.xCtot - q.xCp - q.xCO;
   q.xO = c.xOtot - q.xCO - q.xOp;
   return q;
@@ -679,7 +690,7 @@ template <class F> TCG_FN F dust_T(const CellC<F>& c, F T, F sqT, F guess) {
     F h = c.Bd * y2 * (y2 * y2 - c.Tc4) - c.Gd - C * (T - y);
     if (h > F(0)) hi = y; else lo = y;
     F dh = c.Bd * y * (F(6) * y2 * y2 - F(2) * c.Tc4) + C;
-    F yn = y - m_div(h, dh);
+    F yn = y - h / over(dh);
     const bool newton = (yn >= lo && yn <= hi);  // bracket ends allowed, as above
     if (!newton) yn = F(0.5) * (lo + hi);
     F dy = m_abs(yn - y);
@@ -719,7 +730,7 @@ template <class F, class FC> TCG_FN HRate<F> h_rates(const CellC<FC>& c, const C
 
 template <class F, class FC> TCG_FN F log_psi(const CellC<FC>& c, const ChemT<F>& b, F xe) {
   using K = typename ConstOf<F>::type;
-  return m_log(m_div(c.G0 * b.sqT, m_max(xe * c.n, K(1e-30))) + K(50));
+  return m_log(c.G0 * b.sqT / over(m_max(xe * c.n, K(1e-30))) + K(50));
 }
 
 // ------------------------------------------------------------------ net source terms
@@ -752,10 +763,10 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
   s.CH2 = s.form - s.dest;
   s.CHp = s.ion - s.rec;
   // --- heating per H
-  F eps = m_div(k.eps_num, K(1) + K(0.04996) * m_exp(K(0.431) * lp) * (K(1) + K(0.00430) * m_exp(K(0.692) * lp)));
-  F qH = (K(7.5) + K(24.5) * m_sqrt(m_div(xe, xe + K(0.07)))) * K(EV);
+  F eps = k.eps_num / over(K(1) + K(0.04996) * m_exp(K(0.431) * lp) * (K(1) + K(0.00430) * m_exp(K(0.692) * lp)));
+  F qH = (K(7.5) + K(24.5) * m_sqrt(xe / over(xe + K(0.07)))) * K(EV);
   F dcol = n * (xH * k.fcA + xH2 * k.fcB);
-  F fcol = m_div(dcol, dcol + K(2e-7) + c.zpd);
+  F fcol = dcol / over(dcol + K(2e-7) + c.zpd);
   F G = K(1e-26) * c.G0 * eps * c.Zd                                  // photoelectric
       + c.xi * (xH * qH + K(2) * xH2 * c.qH2)                           // cosmic rays
       + xH * K(3.4 * EV) * c.zpiH + xH2 * K(4.4 * EV) * c.zpiH2         // photoionisation
@@ -773,8 +784,8 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
     // first there.
     F Lrv;
     if constexpr (Prec<F>::fp32_range) Lrv = k.rvLLTE * (nL / den);
-    else Lrv = m_div(k.rvLLTE * nL, den);
-    Lhyd += (den > K(0)) ? m_div(xH2 * Lrv, n) : K(0);
+    else Lrv = k.rvLLTE * nL / over(den);
+    Lhyd += (den > K(0)) ? xH2 * Lrv / over(n) : K(0);
   }
   F Lmet;
   {
@@ -783,7 +794,7 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
     F C01 = C10 * k.cpb;
     // (energies in K; k_B and 1/n applied once at the end, which keeps the partial
     // sums far above FP32's smallest normal number)
-    F lines = q.xCp * m_div(C01, K(2.3e-6) + C10 + C01) * K(2.3e-6 * 91.25);
+    F lines = q.xCp * (C01 / over(K(2.3e-6) + C10 + C01)) * K(2.3e-6 * 91.25);
     // O and C three-level atoms, H and H2 collisions (H2 at half the H rate).  The level
     // populations relative to the ground state are r1 = p1/det and r2 = p2/det, and the
     // cooling per atom (r1 A1 E1 + r2 (A20 E2 + A21 E21)) / (1 + r1 + r2) is taken as
@@ -798,8 +809,8 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
       F det = a11 * a22 - bb * C12o;
       F p1 = C01o * a22 + bb * C02o;
       F p2 = a11 * C02o + C12o * C01o;
-      lines += m_div(q.xO * (p1 * K(8.91e-5 * 227.7) + p2 * K(1.34e-10 * 326.6 + 1.75e-5 * (326.6 - 227.7))),
-                     det + p1 + p2);
+      lines += q.xO * (p1 * K(8.91e-5 * 227.7) + p2 * K(1.34e-10 * 326.6 + 1.75e-5 * (326.6 - 227.7))) /
+               over(det + p1 + p2);
     }
     {
       F C10c = k.ck10 * coll;
@@ -810,17 +821,17 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
       F det = a11 * a22 - bb * C12c;
       F p1 = C01c * a22 + bb * C02c;
       F p2 = a11 * C02c + C12c * C01c;
-      lines += m_div(q.xC * (p1 * K(7.93e-8 * 23.6) + p2 * K(2.0e-14 * 62.4 + 2.65e-7 * (62.4 - 23.6))),
-                     det + p1 + p2);
+      lines += q.xC * (p1 * K(7.93e-8 * 23.6) + p2 * K(2.0e-14 * 62.4 + 2.65e-7 * (62.4 - 23.6))) /
+               over(det + p1 + p2);
     }
-    Lmet = m_div(lines * K(KB), n);
+    Lmet = lines * K(KB) / over(n);
     // CO (stand-in with LVG-like trapping)
-    Lmet += m_div(q.xCO * k.coA, K(1) + m_div(n, k.coN) + q.xCO * c.NtX * K(1e-17));
+    Lmet += q.xCO * k.coA / over(K(1) + n / over(k.coN) + q.xCO * c.NtX * K(1e-17));
     // grain-assisted recombination
     Lmet += k.grT * m_exp(k.grB * lp) * xe * c.Zd;
     // nebular lines (Eq. e:Lambda_neb)
     F ne2 = xe * n * K(0.01);
-    Lmet += m_div(c.Zg * xe * xHp * k.nebT, K(1) + K(0.12) * m_exp(k.nebX * m_log(ne2)));
+    Lmet += c.Zg * xe * xHp * k.nebT / over(K(1) + K(0.12) * m_exp(k.nebX * m_log(ne2)));
     // gas-dust (Eq. eq:gas-dust)
     if constexpr (Prec<F>::cls == 3) s.Td = Td_fixed;  // derivatives: the caller has differentiated the root
     else s.Td = (Td_fixed > K(0)) ? Td_fixed : dust_T(c, b.T, b.sqT, Td_guess);
