@@ -293,12 +293,32 @@ template <class F> struct ChemT {
   F wdH3T, wdHex, wdC3T, wdCex;  // C3 T^C4 and -C5 - C6 ln T for H and C
 };
 
+// The exponentials of the temperature blocks go through `ex(At<i>(), argument)`: ExpPlain
+// evaluates each in place.  Where several lanes hold one cell, the same code runs twice
+// around a shared evaluation: ExpArgs collects the arguments, the lanes evaluate them in
+// turns, ExpVals gives the values (temp_blocks_split in tc_kernels.cuh).  The indices from
+// TEMP_EXPS_SRC on are the equilibrium's.
+template <int I> struct At {};
+struct ExpPlain {
+  template <int I, class G> TCG_FN auto operator()(At<I>, G g) const { return m_exp(g()); }
+};
+constexpr int TEMP_EXPS_SRC = 32, TEMP_EXPS = 38;
+struct ExpArgs {
+  double* a;
+  template <int I, class G> TCG_FN double operator()(At<I>, G g) const { return a[I] = g(), 1.0; }
+};
+struct ExpVals {
+  const double* a;
+  template <int I, class G> TCG_FN double operator()(At<I>, G) const { return a[I]; }
+};
+
 // Electrons of hot gas at log10 T = lt: x_e,He,CIE (two logistic steps, at 4.45 and
 // 4.95, whose exponentials differ by the constant factor exp(0.5/0.06)) + Z'_g
 // x_e,metal,CIE (one step at 5.5).
-template <class F, class FC> TCG_FN F xe_hot_of(const CellC<FC>& c, F lt) {
+template <class F, class FC, class E = ExpPlain>
+TCG_FN F xe_hot_of(const CellC<FC>& c, F lt, E&& ex = E()) {
   using K = typename ConstOf<F>::type;
-  F eHe = m_exp((K(4.45) - lt) * K(1.0 / 0.06));
+  F eHe = ex(At<32>(), [&] { return (K(4.45) - lt) * K(1.0 / 0.06); });
   F xeHe;
   if constexpr (Prec<F>::cls == 0) {  // one quotient (the product stays below 1e70)
     F a = K(1) + eHe, b = K(1) + eHe * K(4160.262005375057);
@@ -306,23 +326,18 @@ template <class F, class FC> TCG_FN F xe_hot_of(const CellC<FC>& c, F lt) {
   } else {
     xeHe = K(0.1) * (K(1) / (K(1) + eHe) + K(1) / (K(1) + eHe * K(4160.262005375057)));  // exp(25/3)
   }
-  F xeMet = K(0.012) * logistic((lt - K(5.5)) * K(4));
+  F xeMet = K(0.012) * (F(1) / over(F(1) + ex(At<33>(), [&] { return -((lt - K(5.5)) * K(4)); })));
   return xeHe + c.Zg * xeMet;
 }
 
 // With `eq` false the factors that only the C/O/e equilibrium takes stay zero: source terms
 // at a given equilibrium (a substep's start, the paper scheme's difference) need 6
 // exponentials and 2 quotients fewer.
-template <class F, class FC> TCG_BIG ChemT<F> chem_T(const CellC<FC>& c, F T, unsigned flags, bool eq = true) {
-  TCG_COUNT(chem_T);
+template <class F, class FC, class E>
+TCG_FN void chem_terms(const CellC<FC>& c, ChemT<F>& b, unsigned flags, bool eq, E&& ex) {
   using K = typename ConstOf<F>::type;
-  ChemT<F> b;
-  b.T = T;
-  b.lnT = m_log(T);
-  b.sqT = m_sqrt(T);
-  const F invT = K(1) / over(T);
-  b.invT = invT;
-  b.S = K(1) / over(K(1) + m_exp(K(-10.0 / 1.5e4) * (T - K(2.75e4))));
+  const F T = b.T, invT = b.invT;
+  b.S = K(1) / over(K(1) + ex(At<0>(), [&] { return K(-10.0 / 1.5e4) * (T - K(2.75e4)); }));
   if (flags & FL_CONST_KGR) {
     b.kgr = K(3.0e-17) * c.Zd;
   } else {
@@ -331,23 +346,39 @@ template <class F, class FC> TCG_BIG ChemT<F> chem_T(const CellC<FC>& c, F T, un
     b.kgr = K(3.0e-17) * c.Zd * K(2) * s2 / over(K(1) + K(0.4) * s2 + K(0.2) * T2 + K(0.08) * T2 * T2);
   }
   F lT4 = b.lnT - K(9.210340371976184);  // ln(T/1e4)
-  b.arr = K(2.54e-13) * m_exp((K(-0.8163) - K(0.0208) * lT4) * lT4);
-  b.kci = K(5.85e-11) * b.sqT * m_exp(K(-157809.1) * invT) / over(K(1) + b.sqT * K(0.003162277660168379));
-  b.kcdH = K(6.67e-12) * b.sqT * m_exp(K(-1) - K(63593.0) * invT);
-  b.kcdH2 = K(5.996e-30) * m_exp(K(4.1881) * b.lnT - K(54657.4) * invT - K(5.6881) * m_log(K(1) + K(6.761e-6) * T));
-  b.wdH3T = K(WDH3) * m_exp(K(WDH4) * b.lnT);
+  b.arr = K(2.54e-13) * ex(At<1>(), [&] { return (K(-0.8163) - K(0.0208) * lT4) * lT4; });
+  b.kci = K(5.85e-11) * b.sqT * ex(At<2>(), [&] { return K(-157809.1) * invT; }) /
+          over(K(1) + b.sqT * K(0.003162277660168379));
+  b.kcdH = K(6.67e-12) * b.sqT * ex(At<3>(), [&] { return K(-1) - K(63593.0) * invT; });
+  b.kcdH2 = K(5.996e-30) * ex(At<4>(), [&] {
+    return K(4.1881) * b.lnT - K(54657.4) * invT - K(5.6881) * m_log(K(1) + K(6.761e-6) * T);
+  });
+  b.wdH3T = K(WDH3) * ex(At<5>(), [&] { return K(WDH4) * b.lnT; });
   b.wdHex = K(-WDH5) - K(WDH6) * b.lnT;
   if (!eq) {
     b.arrC = b.kCpH2 = b.xMH_T = b.xe_hot = b.wdC3T = b.wdCex = F(0);
-    return b;
+    return;
   }
   F lT300 = b.lnT - K(5.703782474656201);  // ln(T/300)
-  b.arrC = K(4.67e-12) * m_exp(K(-0.6) * lT300);
-  b.kCpH2 = K(4.0e-16) * m_exp(K(-0.2) * lT300);
-  b.xMH_T = m_exp(K(0.345) * lT300) * K(2041.2414523193154);  // 1/sqrt(2.4e-7 (T/300)^-0.69)
-  b.xe_hot = xe_hot_of(c, b.lnT * K(0.43429448190325176));  // at log10 T
-  b.wdC3T = K(WDC3) * m_exp(K(WDC4) * b.lnT);
+  b.arrC = K(4.67e-12) * ex(At<34>(), [&] { return K(-0.6) * lT300; });
+  b.kCpH2 = K(4.0e-16) * ex(At<35>(), [&] { return K(-0.2) * lT300; });
+  b.xMH_T = ex(At<36>(), [&] { return K(0.345) * lT300; }) * K(2041.2414523193154);  // 1/sqrt(2.4e-7 (T/300)^-0.69)
+  b.xe_hot = xe_hot_of(c, b.lnT * K(0.43429448190325176), ex);  // at log10 T
+  b.wdC3T = K(WDC3) * ex(At<37>(), [&] { return K(WDC4) * b.lnT; });
   b.wdCex = K(-WDC5) - K(WDC6) * b.lnT;
+}
+template <class F> TCG_FN void temp_powers(ChemT<F>& b, F T) {
+  using K = typename ConstOf<F>::type;
+  b.T = T;
+  b.lnT = m_log(T);
+  b.sqT = m_sqrt(T);
+  b.invT = K(1) / over(T);
+}
+template <class F, class FC> TCG_BIG ChemT<F> chem_T(const CellC<FC>& c, F T, unsigned flags, bool eq = true) {
+  TCG_COUNT(chem_T);
+  ChemT<F> b;
+  temp_powers(b, T);
+  chem_terms(c, b, flags, eq, ExpPlain());
   return b;
 }
 
@@ -370,66 +401,68 @@ template <class F> struct CoolT {
 // temp_blocks_step (which evaluates them afresh at the stepped temperature).
 // Ly-alpha (Eq. e:k_lya): E_21 5.31e-8 T4^0.15 / (1 + (T4/5)^0.65) exp(-11.84/T4) with
 // E_21/k_B = 1.184e5 K, from ln(T/1e4) and 1e4/T.
-template <class F> TCG_FN F lya_of(F lT4, F invT4) {
+template <class F, class E = ExpPlain> TCG_FN F lya_of(F lT4, F invT4, E&& ex = E()) {
   using K = typename ConstOf<F>::type;
-  return K(1.184e5 * KB * 5.31e-8) * m_exp(K(0.15) * lT4 - K(11.84) * invT4) /
-         over(K(1) + m_exp(K(0.65) * (lT4 - K(1.6094379124341003))));
+  return K(1.184e5 * KB * 5.31e-8) * ex(At<6>(), [&] { return K(0.15) * lT4 - K(11.84) * invT4; }) /
+         over(K(1) + ex(At<7>(), [&] { return K(0.65) * (lT4 - K(1.6094379124341003)); }));
 }
 // free-free Gaunt factor at log10 T = lt
-template <class F> TCG_FN F gff_of(F lt) {
+template <class F, class E = ExpPlain> TCG_FN F gff_of(F lt, E&& ex = E()) {
   using K = typename ConstOf<F>::type;
   F dg = K(5.5) - lt;
-  return K(1.1) + K(0.34) * m_exp(-dg * dg * K(1.0 / 3.0));
+  return K(1.1) + K(0.34) * ex(At<8>(), [&] { return -dg * dg * K(1.0 / 3.0); });
 }
 // H2 ro-vibrational LTE rate per molecule from ln(T/1000) and 1000/T (T clamped to
 // [10, 1e4] K by the caller): rotational and vibrational parts
-template <class F> TCG_FN F rovib_lte_of(F lT3, F iT3) {
+template <class F, class E = ExpPlain> TCG_FN F rovib_lte_of(F lT3, F iT3, E&& ex = E()) {
   using K = typename ConstOf<F>::type;
   F q = K(0.13) * iT3;
-  F Lrot = K(9.5e-22) * m_exp(K(3.76) * lT3 - q * q * q) / over(K(1) + K(0.12) * m_exp(K(2.1) * lT3)) +
-           K(3e-24) * m_exp(K(-0.51) * iT3);
-  F Lvib = K(6.7e-19) * m_exp(K(-5.86) * iT3) + K(1.6e-18) * m_exp(K(-11.7) * iT3);
+  F Lrot = K(9.5e-22) * ex(At<9>(), [&] { return K(3.76) * lT3 - q * q * q; }) /
+               over(K(1) + K(0.12) * ex(At<10>(), [&] { return K(2.1) * lT3; })) +
+           K(3e-24) * ex(At<11>(), [&] { return K(-0.51) * iT3; });
+  F Lvib = K(6.7e-19) * ex(At<12>(), [&] { return K(-5.86) * iT3; }) +
+           K(1.6e-18) * ex(At<13>(), [&] { return K(-11.7) * iT3; });
   return Lrot + Lvib;
 }
 // CIE cooling of He and metals (before the S weighting) at log10 T = lt
-template <class F, class FC> TCG_FN F cie_of(const CellC<FC>& c, F lt) {
+template <class F, class FC, class E = ExpPlain> TCG_FN F cie_of(const CellC<FC>& c, F lt, E&& ex = E()) {
   using K = typename ConstOf<F>::type;
   F z1 = (lt - K(5.0)) * K(1.0 / 0.15), z2 = (lt - K(5.35)) * K(1.0 / 0.28), z3 = (lt - K(6.3)) * K(1.0 / 0.35);
-  return K(2.0e-23) * m_exp(K(-0.5) * z1 * z1) +
-         c.Zg * (K(5.4e-22) * m_exp(K(-0.5) * z2 * z2) + K(5.0e-23) * m_exp(K(-0.5) * z3 * z3));
+  return K(2.0e-23) * ex(At<14>(), [&] { return K(-0.5) * z1 * z1; }) +
+         c.Zg * (K(5.4e-22) * ex(At<15>(), [&] { return K(-0.5) * z2 * z2; }) +
+                 K(5.0e-23) * ex(At<16>(), [&] { return K(-0.5) * z3 * z3; }));
 }
 
-template <class F, class FC> TCG_BIG CoolT<F> cool_T(const CellC<FC>& c, const ChemT<F>& b, unsigned flags) {
-  TCG_COUNT(cool_T);
+template <class F, class FC, class E>
+TCG_FN void cool_terms(const CellC<FC>& c, const ChemT<F>& b, CoolT<F>& k, unsigned flags, E&& ex) {
   using K = typename ConstOf<F>::type;
-  CoolT<F> k;
   const F T = b.T, lnT = b.lnT;
   const F invT = b.invT;
-  k.fcA = K(1.0e-12) * b.sqT * m_exp(K(-1000.0) * invT);
-  k.fcB = K(1.4e-12) * b.sqT * m_exp(K(-18100.0) / over(T + K(1200.0)));
-  k.eps_num = K(5.22) + K(2.25) * m_exp(K(0.147) * lnT);
+  k.fcA = K(1.0e-12) * b.sqT * ex(At<17>(), [&] { return K(-1000.0) * invT; });
+  k.fcB = K(1.4e-12) * b.sqT * ex(At<18>(), [&] { return K(-18100.0) / over(T + K(1200.0)); });
+  k.eps_num = K(5.22) + K(2.25) * ex(At<19>(), [&] { return K(0.147) * lnT; });
   F lT4 = lnT - K(9.210340371976184);
   F invT4 = K(1e4) * invT;
-  k.lyaE = lya_of(lT4, invT4);
+  k.lyaE = lya_of(lT4, invT4, ex);
   F lt = lnT * K(0.43429448190325176);
-  k.ffrr = K(1.42e-27) * b.sqT * gff_of(lt) + b.arr * K(KB) * T * (K(0.684) - K(0.0416) * lT4);
+  k.ffrr = K(1.42e-27) * b.sqT * gff_of(lt, ex) + b.arr * K(KB) * T * (K(0.684) - K(0.0416) * lT4);
   // C+ 158 um: n_e,crit = 53 T4^1/2, n_H,crit = 3e3 T2^(-0.1281 - 0.0087 ln T2), A = 2.3e-6
   F lT2 = lnT - K(4.605170185988092);
   k.cpke = K(2.3e-6 / 53.0 * 100.0) * b.sqT * invT;  // / (53 T^1/2 / 100)
-  k.cpkH = K(2.3e-6 / 3e3) * m_exp((K(0.1281) + K(0.0087) * lT2) * lT2);
-  k.cpb = K(2) * m_exp(K(-91.25) * invT);
+  k.cpkH = K(2.3e-6 / 3e3) * ex(At<20>(), [&] { return (K(0.1281) + K(0.0087) * lT2) * lT2; });
+  k.cpb = K(2) * ex(At<21>(), [&] { return K(-91.25) * invT; });
   // O 3-level: n_crit(T) through 2.5e5 (10 K) and 4.9e4 (5000 K); C: 620 and 150
   F lT10 = lnT - K(2.302585092994046);
   const F sO = K(-0.2622274154608984);  // ln(4.9e4/2.5e5)/ln 500
   const F sC = K(-0.22834652828762741);  // ln(150/620)/ln 500
-  k.ok10 = K(8.91e-5 / 2.5e5) * m_exp(-sO * lT10);
+  k.ok10 = K(8.91e-5 / 2.5e5) * ex(At<22>(), [&] { return -sO * lT10; });
   // exp(-E2/T) = exp(-E1/T) exp(-(E2 - E1)/T): two exponentials for the three factors
-  F eO1 = m_exp(K(-227.7) * invT), eO21 = m_exp(K(-(326.6 - 227.7)) * invT);
+  F eO1 = ex(At<23>(), [&] { return K(-227.7) * invT; }), eO21 = ex(At<24>(), [&] { return K(-(326.6 - 227.7)) * invT; });
   k.ob1 = K(3.0 / 5.0) * eO1;
   k.ob2 = K(1.0 / 5.0) * (eO1 * eO21);
   k.ob21 = K(1.0 / 3.0) * eO21;
-  k.ck10 = K(7.93e-8 / 620.0) * m_exp(-sC * lT10);
-  F eC1 = m_exp(K(-23.6) * invT), eC21 = m_exp(K(-(62.4 - 23.6)) * invT);
+  k.ck10 = K(7.93e-8 / 620.0) * ex(At<25>(), [&] { return -sC * lT10; });
+  F eC1 = ex(At<26>(), [&] { return K(-23.6) * invT; }), eC21 = ex(At<27>(), [&] { return K(-(62.4 - 23.6)) * invT; });
   k.cb1 = K(3.0) * eC1;
   k.cb2 = K(5.0) * (eC1 * eC21);
   k.cb21 = K(5.0 / 3.0) * eC21;
@@ -440,29 +473,34 @@ template <class F, class FC> TCG_BIG CoolT<F> cool_T(const CellC<FC>& c, const C
     F lnTc = m_min(m_max(lnT, K(2.302585092994046)), K(9.210340371976184));
     F x = lnTc * K(0.43429448190325176);
     F poly = K(-103.0) + x * (K(97.59) + x * (K(-48.05) + x * (K(10.80) + x * K(-0.9032))));
-    k.rvLlow = m_exp(poly * K(LN10));
+    k.rvLlow = ex(At<28>(), [&] { return poly * K(LN10); });
     F lT3 = lnTc - K(6.907755278982137);
     F iT3;  // 1/T3 = exp(-lT3)
     if constexpr (Prec<F>::cls == 0) iT3 = K(1000) * m_min(m_max(invT, K(1e-4)), K(0.1));
     else iT3 = K(1000) / m_min(m_max(T, K(10)), K(1e4));
-    k.rvLLTE = rovib_lte_of(lT3, iT3);
+    k.rvLLTE = rovib_lte_of(lT3, iT3, ex);
   }
   F st10;
   if constexpr (Prec<F>::cls == 0) st10 = b.sqT * K(0.31622776601683794);
   else st10 = m_sqrt(T * K(0.1));
   k.coA = K(4e-27) * (T * K(0.1)) * st10;
   k.coN = K(3e3) * st10;
-  k.grT = K(4.65e-30) * m_exp(K(0.94) * lnT);
-  k.grB = K(0.74) * m_exp(K(-0.068) * lnT);
+  k.grT = K(4.65e-30) * ex(At<29>(), [&] { return K(0.94) * lnT; });
+  k.grB = K(0.74) * ex(At<30>(), [&] { return K(-0.068) * lnT; });
   F poly = K(6.92e-1) + lT4 * (K(-5.86e-1) + lT4 * (K(8.16e-1) + lT4 * (K(-5.05e-1) +
            lT4 * (K(1.18e-1) + lT4 * (K(7.66e-3) + lT4 * K(-5.08e-3))))));
-  k.nebT = K(3.68e-23) * m_exp(poly * K(LN10) - K(3.86) * invT4 - K(0.5) * lT4);
+  k.nebT = K(3.68e-23) * ex(At<31>(), [&] { return poly * K(LN10) - K(3.86) * invT4 - K(0.5) * lT4; });
   k.nebX = K(0.38) - K(0.12) * lT4;
   if (flags & FL_NO_CIE) {
     k.cie = K(0);
   } else {
-    k.cie = cie_of(c, lt);
+    k.cie = cie_of(c, lt, ex);
   }
+}
+template <class F, class FC> TCG_BIG CoolT<F> cool_T(const CellC<FC>& c, const ChemT<F>& b, unsigned flags) {
+  TCG_COUNT(cool_T);
+  CoolT<F> k;
+  cool_terms(c, b, k, flags, ExpPlain());
   return k;
 }
 
