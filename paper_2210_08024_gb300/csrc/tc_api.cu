@@ -365,6 +365,20 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
   return Shape{(int)g, b, lpc, groups, chosen};
 }
 
+// Cells dealt to the warps of a cooperative launch, rank r of the cost order to warp r mod
+// warps, instead of claimed from the queue; 0: none.  Where every cell has its own lanes, the
+// launch lasts as long as its slowest warp, and a queue hands the longest cells to one warp,
+// whose lanes wait for one another throughout.  Queue / dealt, ms: FP64 Newton, 4800 slab cells
+// over 1e3 yr 2.34 / 1.94, stiff cells 3.18 / 2.47, 1500 slab cells over 1e4 yr 3.61 / 3.26, 1000
+// over 100 yr 0.82 / 0.70, 4096 random states over 1e4 yr 36.2 / 30.9 (4800 over 100 yr 14.8 /
+// 16.2); mixed, 1500 slab cells over 1e4 yr 3.75 / 3.28, 4800 random states 32.3 / 33.9.  A cost
+// hint orders by the cost itself: alike cells then share a warp and its code (the PDR driver's
+// 48 x 100 cells 122 / 162 ms), so those and the drivers' first chunks stay with the queue.
+static int dealt_cells(const Shape& sh, long long ntotal) {
+  const long long slots = (long long)sh.grid * sh.block / 32 * sh.groups;
+  return (sh.lpc == 4 && ntotal <= slots) ? (int)slots : 0;
+}
+
 // Grows the cost-ordering workspace to ncell cells (not while `st` is being captured).
 // Returns false if there is none to use.
 static bool order_workspace(tc_handle* h, long long ncell, cudaStream_t st) {
@@ -392,7 +406,8 @@ static bool order_workspace(tc_handle* h, long long ncell, cudaStream_t st) {
   return true;
 }
 
-static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long ntotal, double dt, cudaStream_t st) {
+static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long ntotal, double dt, cudaStream_t st,
+                   bool deal = true) {
   int kmode = kernel_mode(h->p.mode);
   if (h->p.mode == TC_MODE_MIXED_SEEDED || h->p.mode == TC_MODE_NEWTON_FP64_SEEDED) {
     if (!h->d_mlp) return TC_ENOMLP;
@@ -410,6 +425,7 @@ static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long 
       return TC_ECUDA;
     h->launches += 3;
     dp.order = h->d_order;
+    if (deal && !f.hint) dp.deal = dealt_cells(sh, ntotal);
   }
   cudaError_t e;
   if (sh.lpc == 4 && kmode == 1) e = tcg::launch_mode1_coop(f, dp, dt, h->d_cursor, ntotal, grid, block, st);
@@ -856,7 +872,7 @@ extern "C" int tc_eq_curves(tc_handle* h, const tc_eq_spec* s, const tc_eq_out* 
       return TC_ECUDA;
     h->launches += 1;
     f.hint = (k > 0) ? f.iters : nullptr;  // order each chunk by the previous chunk's iterations
-    int rc = enqueue(h, false, f, ncell, dt, st);
+    int rc = enqueue(h, false, f, ncell, dt, st, false);
     if (rc != TC_OK) return rc;
   }
   if (tcg::launch_eq_finish(g, w, o->T, o->x_h2, o->x_hp, o->x_e, o->P_k, o->chg, o->status, st) != cudaSuccess)
@@ -930,7 +946,7 @@ extern "C" int tc_pdr(tc_handle* h, const tc_pdr_spec* s, const tc_pdr_out* o, v
       return TC_ECUDA;
     h->launches += 1;
     f.hint = (k > 0) ? f.iters : nullptr;  // order each chunk by the previous chunk's iterations
-    int rc = enqueue(h, false, f, ncell, dt, st);
+    int rc = enqueue(h, false, f, ncell, dt, st, false);
     if (rc != TC_OK) return rc;
   }
   if (tcg::launch_pdr_fields(g, w, o->T, o->x_h2, o->x_hp, s->nchunk, true, o->chi_pe, o->f_shld_h2, o->N_c, st) !=

@@ -598,10 +598,10 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 //     thousandfold).  Two evaluations usually do.
 // Converged when every step is below rtol |y_i| as in newton_iter, or one step earlier,
 // when two steps in a row show that the next would lie far below it: with rho = d_k /
-// d_(k-1), what remains after step k is at most ~rho d_k, accepted below 1e-2 rtol (2-norm
+// d_(k-1), what remains after step k is at most ~rho d_k, accepted below 1e-2 rtol.  The C/O/e
+// equilibrium of the last evaluation is moved along the last step by its derivatives.  2-norm
 // errors on 20,000 slab cells against roots solved to rounding: T 1.1e-16, x_e 1.8e-16; by the
-// plain iteration 3.9e-15, 4.7e-14).  The C/O/e
-// equilibrium of the last evaluation is moved along the last step by its derivatives.
+// plain iteration 3.9e-15, 4.7e-14.
 //
 // Returns the iterations of both phases, or -1 when a step would have to be damped, fails to
 // shrink by half or is not finite, or when TAN_MAXIT iterations pass; the plain solver then
@@ -1515,9 +1515,17 @@ __global__ void __launch_bounds__(step_threads(MODE, LPC),
   bool have = false;
   // the work queue is empty for this lane, or the lane's group of a sparse warp takes no cells
   bool done = LPC > 1 && (int)((threadIdx.x & 31u) / LPC) >= p.groups;
+  bool deal = LPC > 1 && p.deal > 0;  // the first cell is dealt, not claimed
   while (true) {
     if (!have && !done) {
-      long long gi = claim_cells_lpc<LPC>(cursor);
+      long long gi;
+      if (LPC > 1 && deal) {
+        const unsigned nw = gridDim.x * (blockDim.x >> 5), w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        gi = (long long)((threadIdx.x & 31u) / LPC) * nw + w;
+        deal = false;
+      } else {
+        gi = claim_cells_lpc<LPC>(cursor) + ((LPC > 1) ? p.deal : 0);
+      }
       if (gi >= ntotal) {
         done = true;
       } else {

@@ -173,6 +173,7 @@ struct DevParams {
   unsigned flags;
   const unsigned* order = nullptr;  // optional: the k-th claimed cell is order[k] (cost-ordered queue)
   int groups = 8;  // cooperative kernels: cells a warp advances at once (of 32 / lanes per cell)
+  int deal = 0;    // cooperative kernels: cells dealt over the warps before the queue, which goes on there, or 0
   const MlpMma* mlp_mma = nullptr;  // seeded modes: the network for the warp-level inference
 };
 
