@@ -89,7 +89,7 @@ __device__ __forceinline__ float silu_d(float z) {
 // 128 SMs.
 constexpr int TS = 64;          // samples per tile
 constexpr int LD = TS + 4;      // row length of an activation
-constexpr int NT = 256;         // threads per block
+constexpr int NT = 256;         // threads per block (eight warps)
 constexpr int HID = MLP_HID;
 static_assert(HID == 64 && MLP_OUT == 3 && MLP_IN <= 16, "thread maps below");
 
@@ -183,13 +183,18 @@ __device__ __forceinline__ void layer_dw(const float* __restrict__ G, const floa
 }
 
 // The forward pass of B rows of X (out, when given, receives the outputs), and with TRAIN
-// the loss sum_b sum_m w_m (O - Y)^2 / B and its gradient, both added to what grad and loss
-// hold.
+// the loss sum_b sum_m w_m (O - Y)^2 / B, and its gradient added to what grad holds.  The loss
+// of the blocks is summed in FP64 (acc, zero at the start) and written by the last one: FP32
+// additions of the 768 warps' sums to one word left it up to 1.6e-6 off.
+struct LossAcc {
+  double sum;
+  unsigned blocks;
+};
 template <bool TRAIN>
 __global__ void __launch_bounds__(NT) k_pass(const float* __restrict__ theta, const float* __restrict__ norm,
                                              const float* __restrict__ X, const float* __restrict__ Y, int B, float w0,
                                              float w1, float w2, float* __restrict__ out, float* __restrict__ grad,
-                                             float* __restrict__ loss) {
+                                             LossAcc* __restrict__ acc, float* __restrict__ loss) {
   extern __shared__ float4 smem_raw[];
   Smem& m = *reinterpret_cast<Smem*>(smem_raw);
   const int t = threadIdx.x;
@@ -274,6 +279,18 @@ __global__ void __launch_bounds__(NT) k_pass(const float* __restrict__ theta, co
     }
   }
   if (!TRAIN) return;
+  __shared__ float ws[NT / 32];
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+  if ((t & 31) == 0) ws[t >> 5] = lsum;
+  __syncthreads();
+  if (t == 0) {
+    atomicAdd(&acc->sum, (double)(((ws[0] + ws[1]) + (ws[2] + ws[3])) + ((ws[4] + ws[5]) + (ws[6] + ws[7]))));
+    __threadfence();
+    if (loss && atomicAdd(&acc->blocks, 1u) == gridDim.x - 1) {
+      __threadfence();
+      *loss = (float)atomicAdd(&acc->sum, 0.0);
+    }
+  }
   {
     const int kx = t & 15, n0 = 4 * (t >> 4);
 #pragma unroll
@@ -298,8 +315,6 @@ __global__ void __launch_bounds__(NT) k_pass(const float* __restrict__ theta, co
       if (k0 + 4 * j < MLP_IN) atomicAdd(grad + OFF_W1 + n * MLP_IN + k0 + 4 * j, dw1[j]);
     if (k0 == 0) atomicAdd(grad + OFF_B1 + n, db1);
   }
-  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
-  if ((t & 31) == 0 && lsum != 0.f) atomicAdd(loss, lsum);
 }
 
 __global__ void k_adam(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
@@ -324,7 +339,7 @@ struct tc_mlp {
   float* m = nullptr;
   float* v = nullptr;
   float* norm = nullptr;   // mean[MLP_IN], inv_std[MLP_IN]
-  float* loss = nullptr;
+  LossAcc* acc = nullptr;
   int num_sms = 1;
   long long t = 0;         // Adam step count
   float h_mean[MLP_IN], h_inv_std[MLP_IN];
@@ -360,7 +375,7 @@ int tc_mlp_create(unsigned long long seed, tc_mlp** out) {
             cudaMalloc(&h->m, NPARAM * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&h->v, NPARAM * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&h->norm, 2 * MLP_IN * sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&h->loss, sizeof(float)) == cudaSuccess;
+            cudaMalloc(&h->acc, sizeof(LossAcc)) == cudaSuccess;
   int dev = 0;
   ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
        cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
@@ -409,7 +424,7 @@ void tc_mlp_destroy(tc_mlp* h) {
   cudaFree(h->m);
   cudaFree(h->v);
   cudaFree(h->norm);
-  cudaFree(h->loss);
+  cudaFree(h->acc);
   delete h;
 }
 
@@ -442,7 +457,7 @@ int tc_mlp_predict(tc_mlp* h, const float* X, int B, float* out, void* stream) {
   if (!h || B < 0 || (B > 0 && (!X || !out))) return TC_EINVAL;
   if (B == 0) return TC_OK;
   k_pass<false><<<pass_grid(h, B), NT, sizeof(Smem), (cudaStream_t)stream>>>(h->theta, h->norm, X, nullptr, B, 0.f, 0.f,
-                                                                             0.f, out, nullptr, nullptr);
+                                                                             0.f, out, nullptr, nullptr, nullptr);
   return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
 }
 
@@ -451,11 +466,10 @@ int tc_mlp_grad(tc_mlp* h, const float* X, const float* Y, int B, const float* w
   if (!h || B < 1 || !X || !Y) return TC_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   float* g = grad ? grad : h->grad;
-  float* l = loss ? loss : h->loss;
   if (cudaMemsetAsync(g, 0, NPARAM * sizeof(float), st) != cudaSuccess) return TC_ECUDA;
-  if (cudaMemsetAsync(l, 0, sizeof(float), st) != cudaSuccess) return TC_ECUDA;
+  if (cudaMemsetAsync(h->acc, 0, sizeof(LossAcc), st) != cudaSuccess) return TC_ECUDA;
   const float w0 = w3 ? w3[0] : 1.f, w1 = w3 ? w3[1] : 1.f, w2 = w3 ? w3[2] : 1.f;
-  k_pass<true><<<pass_grid(h, B), NT, sizeof(Smem), st>>>(h->theta, h->norm, X, Y, B, w0, w1, w2, nullptr, g, l);
+  k_pass<true><<<pass_grid(h, B), NT, sizeof(Smem), st>>>(h->theta, h->norm, X, Y, B, w0, w1, w2, nullptr, g, h->acc, loss);
   return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
 }
 
