@@ -43,14 +43,13 @@ UNIT = "cell-updates/s"
 FP64_NOMINAL_TFLOPS = 1.25
 
 STATE_KEYS = ("T", "xH2", "xHp")
-# DRAM bytes per cell of one k_step<1> launch on the 128^3 slab in the benchmark's
-# autotuned shape (64 threads x 1824 blocks, 768 resident threads per SM), from ncu
-# (dram__bytes_read.sum + dram__bytes_write.sum, one pass,
-# profiles/k_step_fp64_slab128.md): 20.07 GB read + 29.21 GB written for 2,097,152
-# cells.  Almost all of it is the per-thread stack (spills at the 80-register cap and
-# the structs passed to the out-of-line physics): ~3 KB per thread for 768 resident
-# threads per SM is ~350 MB, almost three times L2.  The cells' own data are 152 B.
-TRAFFIC_BYTES_PER_CELL = 23499.0
+# DRAM bytes per cell of one k_step<1> launch on the 128^3 slab in the default shape (128
+# threads x 1216 blocks, 1024 resident threads per SM), from ncu (dram__bytes_read.sum +
+# dram__bytes_write.sum, one pass, profiles/step_counters.md): 13.49 GB read + 22.46 GB
+# written for 2,097,152 cells.  Almost all of it is the per-thread stack (spills at the
+# 64-register cap and the structs passed to the out-of-line physics), whose sum over the
+# resident threads exceeds L2.  The cells' own data are 152 B.
+TRAFFIC_BYTES_PER_CELL = 17145.0
 
 
 def parse():
@@ -444,12 +443,12 @@ def run_onezone(args, tc, torch, stream):
     return res
 
 
-# FP64 operations per cell of tc_sixray, counted from the kernel source: per ray the
-# H2 self-shielding factor (4 divides, a square root, an exponential), the ray weight
-# (an exponential and a square root) and ~15 adds/multiplies with the scans; per cell
-# the two cell averages (expm1 and a divide each), the two fields (an exponential each),
-# f_shld,H2 and N_eff (a divide each, a logarithm), the CR rate and the two chi0/6 (a divide each).
-SIXRAY_OPS = {"add": 50.0, "mul": 40.0, "div": 31.0, "sqrt": 12.0, "exp": 16.0, "log": 1.0}
+# FP64 operations per cell of tc_sixray, counted from the kernel source (an FMA as an add and
+# a multiply): per ray the columns and their arguments, the H2 self-shielding factor (one
+# exponential, 20 FMAs and multiplies) and, but for a cell's first ray, the weight (one
+# exponential, 10 FMAs and multiplies); per cell the two cell averages (19 FMAs each), the two
+# fields (an exponential each), f_shld,H2 and the CR rate (a divide each) and N_eff (a logarithm).
+SIXRAY_OPS = {"add": 160.0, "mul": 232.0, "div": 2.0, "sqrt": 0.0, "exp": 13.0, "log": 1.0}
 
 
 def run_sixray(args, tc, torch, stream, peaks):

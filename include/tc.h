@@ -94,13 +94,12 @@ typedef struct tc_params {
   int lanes_per_cell;          /* lanes that advance one cell together (the library's scheduling, no
                                   counterpart in the paper; results agree to rounding): 1, or 4 for the
                                   warp-cooperative kernels of modes TC_MODE_NEWTON_FP64 and TC_MODE_MIXED,
-                                  whose four lanes evaluate the four points of each forward-difference
-                                  Jacobian at once (tc_step and tc_step_host only; other modes and
-                                  tc_step_batch use 1).  0 (default): for TC_MODE_NEWTON_FP64 and
+                                  whose four lanes split each Jacobian (derivative directions, or points
+                                  of a forward difference) and share FP64 exponentials (tc_step and
+                                  tc_step_host only; other modes and tc_step_batch use 1).  0 (default): for TC_MODE_NEWTON_FP64 and
                                   TC_MODE_MIXED 4 on launches too small to fill the GPU, whose time is
                                   the latency of the slowest cells (up to 64 and 32 cells per SM), else
-                                  1, unless
-                                  tc_autotune has recorded a choice for the launch's size class. */
+                                  1, unless tc_autotune has recorded a choice for the launch's size class. */
 } tc_params;
 
 typedef struct tc_fields {

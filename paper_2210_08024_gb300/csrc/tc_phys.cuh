@@ -14,7 +14,7 @@
 // its cell constants in FP32 (type FC, elsewhere the same as F).  Terms
 // the paper names but does not print (closures: cited fits and tables it does not
 // reproduce) use one stated definition each, labelled where it is a stand-in for the
-// cited source; the CPU checker uses the same definitions, written independently.
+// cited source; the CPU oracle uses the same definitions, written independently.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>

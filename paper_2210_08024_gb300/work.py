@@ -144,7 +144,7 @@ def main(sample: int = 8192):
 
 # FMA-slot cost per operation class, as tc_peak measures it on a GB300 (the benchmark
 # measures them again in each run; these are the values of one run, for the breakdown)
-SLOT_WEIGHTS = {"add": 1.0, "mul": 1.0, "div": 5.67, "sqrt": 8.61, "exp": 16.0, "log": 30.2}
+SLOT_WEIGHTS = {"add": 1.0, "mul": 1.0, "div": 5.67, "sqrt": 8.62, "exp": 10.8, "log": 20.9}
 
 
 def breakdown(res: dict, mode: str = "mode1") -> list:
