@@ -17,7 +17,7 @@ LIB = os.path.join(HERE, "libtc_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["tc_api.cu", "tc_onezone.cu", "tc_sixray.cu", "tc_pdr.cu", "tc_order.cu", "tc_k_paper.cu", "tc_k_newton.cu", "tc_k_mixed.cu", "tc_mlp.cu", "tc_peak.cu",
            "tc_static.cu", "tc_k_seeded3.cu", "tc_k_seeded4.cu", "tc_k_newton_coop.cu", "tc_k_mixed_coop.cu",
-           "tc_df64_diag.cu"]
+           "tc_df64_diag.cu", "tc_k_driver_paper.cu", "tc_k_driver_newton.cu", "tc_k_driver_seeded4.cu"]
 
 
 def nvcc() -> str:

@@ -257,7 +257,11 @@ static int kernel_mode(int mode) {
   }
 }
 
-static int coop_occupancy(int kmode, int block) {
+// Whether a driver's launch takes the drivers' own kernels: the FP64 modes.
+static bool driver_kernel(int kmode, bool driver) { return driver && (kmode == 0 || kmode == 1 || kmode == 4); }
+
+static int coop_occupancy(int kmode, int block, bool driver = false) {
+  if (driver_kernel(kmode, driver)) return tcg::occupancy_driver1_coop(block);
   return (kmode == 1) ? tcg::occupancy_mode1_coop(block) : tcg::occupancy_mode2_coop(block);
 }
 
@@ -312,6 +316,14 @@ static bool default_coop(int kmode, long long ntotal, int num_sms) {
   return ntotal <= (long long)num_sms * 32 * ((kmode == 1) ? 2 : 1);
 }
 
+// The same for the drivers: four lanes while every cell's fit the resident lanes (19,456 cells).  A
+// cell's results on one and on four lanes differ by rounding (mode 1) or by the polish's
+// remainder (mode 2), which a driver's chunks can multiply (tc_k_driver.cuh), so this line lies
+// where it has always lain.
+static bool driver_coop(int kmode, long long ntotal, int num_sms) {
+  return ntotal * 4 <= (long long)num_sms * coop_occupancy(kmode, 128, true) * 128;
+}
+
 // Cells that a warp of the cooperative kernels advances at once: eight, or fewer where that
 // leaves SM partitions without a warp (lanes of one warp wait for one another; random states,
 // mode 1, ms with 8 / 4 / 2 / 1 cells a warp: 500 cells 32 / 27 / 27 / 25, 2000 33 / 30 / 34 / 37,
@@ -321,7 +333,7 @@ static int coop_groups(long long ntotal, int num_sms) {
   return (g < 1) ? 1 : (g > 8) ? 8 : (int)g;
 }
 
-static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal) {
+static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal, bool driver = false) {
   int b = h->p.block, per_sm = h->p.blocks_per_sm, lpc = h->p.lanes_per_cell;
   const bool coop_ok = (kmode == 1 || kmode == 2) && !batch;
   const tc_handle::Tuned& t = h->tuned[size_class(ntotal)];
@@ -336,7 +348,8 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
   b = (b / 32) * 32;
   if (b < 32) b = 32;
   if (!coop_ok) lpc = 1;
-  if (lpc <= 0) lpc = (coop_ok && default_coop(kmode, ntotal, h->num_sms)) ? 4 : 1;
+  if (lpc <= 0)
+    lpc = (coop_ok && (driver ? driver_coop(kmode, ntotal, h->num_sms) : default_coop(kmode, ntotal, h->num_sms))) ? 4 : 1;
   if (lpc != 4) lpc = 1;
   if (auto_block) {
     int ps = 0;
@@ -351,7 +364,10 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal)
   }
   const int chosen = per_sm > 0 ? per_sm : 0;
   if (per_sm <= 0) {
-    per_sm = (lpc == 4) ? coop_occupancy(kmode, b)
+    per_sm = (lpc == 4)                      ? coop_occupancy(kmode, b, driver)
+             : driver_kernel(kmode, driver) ? ((kmode == 0)   ? tcg::occupancy_driver0(b)
+                                               : (kmode == 1) ? tcg::occupancy_driver1(b)
+                                                              : tcg::occupancy_driver4(b))
              : (kmode == 0) ? tcg::occupancy_mode0_impl(b)
              : (kmode == 1) ? tcg::occupancy_mode1_impl(b)
              : (kmode == 2) ? tcg::occupancy_mode2_impl(b)
@@ -407,12 +423,12 @@ static bool order_workspace(tc_handle* h, long long ncell, cudaStream_t st) {
 }
 
 static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long ntotal, double dt, cudaStream_t st,
-                   bool deal = true) {
+                   bool driver = false) {
   int kmode = kernel_mode(h->p.mode);
   if (h->p.mode == TC_MODE_MIXED_SEEDED || h->p.mode == TC_MODE_NEWTON_FP64_SEEDED) {
     if (!h->d_mlp) return TC_ENOMLP;
   }
-  const Shape sh = launch_shape(h, kmode, batch, ntotal);
+  const Shape sh = launch_shape(h, kmode, batch, ntotal, driver);
   const int grid = sh.grid, block = sh.block;
   if (cudaMemsetAsync(h->d_cursor, 0, sizeof(unsigned long long), st) != cudaSuccess) return TC_ECUDA;
   tcg::DevParams dp = dev_params(h->p);
@@ -425,10 +441,16 @@ static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long 
       return TC_ECUDA;
     h->launches += 3;
     dp.order = h->d_order;
-    if (deal && !f.hint) dp.deal = dealt_cells(sh, ntotal);
+    if (!driver && !f.hint) dp.deal = dealt_cells(sh, ntotal);
   }
   cudaError_t e;
-  if (sh.lpc == 4 && kmode == 1) e = tcg::launch_mode1_coop(f, dp, dt, h->d_cursor, ntotal, grid, block, st);
+  if (driver_kernel(kmode, driver)) {
+    const auto launch = (sh.lpc == 4)   ? tcg::launch_driver1_coop
+                        : (kmode == 0) ? tcg::launch_driver0
+                        : (kmode == 1) ? tcg::launch_driver1
+                                       : tcg::launch_driver4;
+    e = launch(f, dp, dt, h->d_cursor, ntotal, grid, block, st);
+  } else if (sh.lpc == 4 && kmode == 1) e = tcg::launch_mode1_coop(f, dp, dt, h->d_cursor, ntotal, grid, block, st);
   else if (sh.lpc == 4 && kmode == 2) e = tcg::launch_mode2_coop(f, dp, dt, h->d_cursor, ntotal, grid, block, st);
   else if (kmode == 0) e = tcg::launch_mode0(batch, f, h->d_boxes, dp, dt, h->d_cursor, ntotal, grid, block, st);
   else if (kmode == 1) e = tcg::launch_mode1(batch, f, h->d_boxes, dp, dt, h->d_cursor, ntotal, grid, block, st);
@@ -872,7 +894,7 @@ extern "C" int tc_eq_curves(tc_handle* h, const tc_eq_spec* s, const tc_eq_out* 
       return TC_ECUDA;
     h->launches += 1;
     f.hint = (k > 0) ? f.iters : nullptr;  // order each chunk by the previous chunk's iterations
-    int rc = enqueue(h, false, f, ncell, dt, st, false);
+    int rc = enqueue(h, false, f, ncell, dt, st, true);
     if (rc != TC_OK) return rc;
   }
   if (tcg::launch_eq_finish(g, w, o->T, o->x_h2, o->x_hp, o->x_e, o->P_k, o->chg, o->status, st) != cudaSuccess)
@@ -946,7 +968,7 @@ extern "C" int tc_pdr(tc_handle* h, const tc_pdr_spec* s, const tc_pdr_out* o, v
       return TC_ECUDA;
     h->launches += 1;
     f.hint = (k > 0) ? f.iters : nullptr;  // order each chunk by the previous chunk's iterations
-    int rc = enqueue(h, false, f, ncell, dt, st, false);
+    int rc = enqueue(h, false, f, ncell, dt, st, true);
     if (rc != TC_OK) return rc;
   }
   if (tcg::launch_pdr_fields(g, w, o->T, o->x_h2, o->x_hp, s->nchunk, true, o->chi_pe, o->f_shld_h2, o->N_c, st) !=

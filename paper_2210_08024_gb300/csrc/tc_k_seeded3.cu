@@ -2,7 +2,7 @@
 // FP64 runs only in this kernel's rare fallbacks: exp() and log() keep its code, bound by
 // instruction fetch, as it was (with the tables of tc_exp64.cuh the seeded mixed step on the
 // 128^3 slab took 55.5 ms against 51.5).
-#define TCG_PLAIN_EXP64
+#define TCG_PLAIN_FP64
 #include "tc_k_seeded.cuh"
 
 namespace tcg {

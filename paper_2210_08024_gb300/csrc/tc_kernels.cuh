@@ -1135,7 +1135,11 @@ TCG_FN void substep_newton64(const CellC<double>& c, const CellC<float>& cf, con
   bool last;
   double src[3];
   const double dts = substep_start64<LPC>(c, p, dt, s, td_g, last, src);
+#ifdef TCG_DRIVER
+  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g);  // by the plain iteration
+#else
   solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, src);
+#endif
 }
 template <int LPC = 1>
 TCG_FN void substep_newton64(const CellC<double>& c, const DevParams& p, double dt, LaneState& s, double& xe_g,
@@ -1469,6 +1473,7 @@ TCG_FN bool seed_from_outputs(const float* o, const double* g, const LaneState& 
 // (293.5 ms; 300.1 at 6).
 constexpr int STEP_MIN_BLOCKS = 8;
 constexpr int STEP_MIN_BLOCKS_PAPER = 4;
+constexpr int STEP_MIN_BLOCKS_DRIVER = 6;  // mode 1 by the plain iteration (4 / 5 / 6: 214.1 / 213.3 / 212.9 ms)
 // The warp-cooperative kernels (four lanes per cell) serve launches too small to fill
 // the GPU, where the time is the latency of the slowest cells: 4 resident blocks (128
 // registers per thread) spill less.
@@ -1490,14 +1495,27 @@ constexpr int step_threads(int mode, int lpc) {
   return (lpc == 1 && (mode == 2 || mode == 3)) ? STEP_THREADS_MIXED : STEP_THREADS;
 }
 
-template <int MODE, bool BATCH, int LPC = 1>
-__global__ void __launch_bounds__(step_threads(MODE, LPC),
-                                  (LPC == 1) ? ((MODE == 2 || MODE == 3) ? STEP_MIN_BLOCKS_MIXED
-                                                : (MODE == 0)            ? STEP_MIN_BLOCKS_PAPER
-                                                                         : STEP_MIN_BLOCKS)
-                                             : STEP_MIN_BLOCKS_COOP)
+// The kernels of the equilibrium and PDR drivers, instantiated as mode DRIVER + m for m = 0, 1
+// and 4 (tc_k_driver.cuh).
+constexpr int DRIVER = 8;
+constexpr int step_min_blocks(int kmode, int lpc) {
+  return (lpc != 1)                        ? STEP_MIN_BLOCKS_COOP
+         : (kmode == 2 || kmode == 3)      ? STEP_MIN_BLOCKS_MIXED
+         : (kmode % DRIVER == 0)           ? STEP_MIN_BLOCKS_PAPER
+         : (kmode == DRIVER + 1)           ? STEP_MIN_BLOCKS_DRIVER
+                                           : STEP_MIN_BLOCKS;
+}
+
+template <int KMODE, bool BATCH, int LPC = 1>
+__global__ void __launch_bounds__(step_threads(KMODE, LPC), step_min_blocks(KMODE, LPC))
     k_step(DevFields f1, const BoxTable* __restrict__ boxes, DevParams p, double dt, unsigned long long* cursor,
            long long ntotal, const MlpDev* __restrict__ mlp) {
+  constexpr int MODE = KMODE % DRIVER;
+#ifdef TCG_DRIVER
+  static_assert(KMODE >= DRIVER, "driver kernels only");
+#else
+  static_assert(KMODE < DRIVER, "the driver kernels have their own translation units");
+#endif
   static_assert(LPC == 1 || ((MODE == 1 || MODE == 2) && !BATCH), "cooperative kernels: modes 1 and 2, one box");
   constexpr bool SEEDED = (MODE == 3 || MODE == 4);
   constexpr bool MIXED = (MODE == 2 || MODE == 3);
@@ -1622,7 +1640,7 @@ __global__ void __launch_bounds__(step_threads(MODE, LPC),
       }
     } else {
       // modes 1 and 2 with one lane per cell: threads stay until their block is done
-      constexpr bool SYNC = (MODE == 1 || MODE == 2) && LPC == 1;
+      constexpr bool SYNC = (KMODE == 1 || KMODE == 2) && LPC == 1;
       if constexpr (SYNC) {
         if (__syncthreads_and(done)) break;
       } else {

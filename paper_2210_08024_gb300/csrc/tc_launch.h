@@ -27,6 +27,19 @@ cudaError_t launch_mode3(bool batch, const DevFields& f, const BoxTable* d_boxes
 cudaError_t launch_mode4(bool batch, const DevFields& f, const BoxTable* d_boxes, const DevParams& p, double dt,
                          unsigned long long* cursor, long long ntotal, int grid, int block, cudaStream_t st,
                          const MlpDev* mlp);
+// The drivers' kernels of the FP64 modes (tc_k_driver.cuh), one lane per cell or, of mode 1, four.
+cudaError_t launch_driver0(const DevFields& f, const DevParams& p, double dt, unsigned long long* cursor,
+                           long long ntotal, int grid, int block, cudaStream_t st);
+int occupancy_driver0(int block);
+cudaError_t launch_driver1(const DevFields& f, const DevParams& p, double dt, unsigned long long* cursor,
+                           long long ntotal, int grid, int block, cudaStream_t st);
+int occupancy_driver1(int block);
+cudaError_t launch_driver1_coop(const DevFields& f, const DevParams& p, double dt, unsigned long long* cursor,
+                           long long ntotal, int grid, int block, cudaStream_t st);
+int occupancy_driver1_coop(int block);
+cudaError_t launch_driver4(const DevFields& f, const DevParams& p, double dt, unsigned long long* cursor,
+                           long long ntotal, int grid, int block, cudaStream_t st);
+int occupancy_driver4(int block);
 // Device check of the df64 source terms (tc_df64_diag.cu; tc_df64_source_check).
 cudaError_t launch_df64_source_check(const DevFields& f, const DevParams& p, double* err, cudaStream_t st);
 }  // namespace tcg

@@ -23,6 +23,13 @@
 #include "tc_df64.cuh"
 #include "tc_exp64.cuh"
 
+// TCG_PLAIN_FP64: device FP64 by CUDA's exp(), log() and division, each quotient on its own and
+// inner roots to rounding.  The mixed kernels' translation units define it (FP64 runs only in
+// their rare fallbacks), and those of the drivers' kernels (TCG_DRIVER, tc_k_driver.cuh).
+#ifdef TCG_DRIVER
+#define TCG_PLAIN_FP64
+#endif
+
 // Physics and substep functions are host+device so the host compiler can also build
 // them (used by the host-side test harness of the library's own kernels).
 #ifndef TCG_FN
@@ -68,7 +75,7 @@ constexpr unsigned FL_CONST_KGR = 1u, FL_NO_ROVIB = 2u, FL_NO_CIE = 4u;
 // line: the physics blocks hold ~50 call sites, and one shared copy keeps the kernels' code
 // smaller (instruction fetch; with exp() and log() out of line the FP64 Newton step on the
 // 128^3 slab took 226.5 ms, inlined 232.5).
-#ifdef TCG_PLAIN_EXP64
+#ifdef TCG_PLAIN_FP64
 __device__ __noinline__ static double m_exp64_ool(double x) { return exp(x); }
 __device__ __noinline__ static double m_log64_ool(double x) { return log(x); }
 #else
@@ -105,7 +112,7 @@ TCG_FN float m_abs(float a) { return fabsf(a); }
 // below 0.51 ulp (tests/test_gpu_div64.py).  Exponents from which a step could leave the range
 // take the plain division.
 TCG_FN double m_div(double a, double b) {
-#if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_EXP64)
+#if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_FP64)
   if ((unsigned)((hi_word(b) & 0x7fffffff) - 0x10000000) < 0x60000000u &&
       (unsigned)(hi_word(a) & 0x7fffffff) < 0x70000000u) {
     double y;
@@ -127,7 +134,7 @@ struct OverF64 {
 };
 TCG_FN double operator/(double a, OverF64 d) { return m_div(a, d.b); }
 template <class F> TCG_FN F over(F b) { return b; }
-#if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_EXP64)
+#if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_FP64)
 TCG_FN OverF64 over(double b) { return OverF64{b}; }
 #endif
 
@@ -151,6 +158,13 @@ template <> struct Prec<df64> {
   static constexpr bool fp32_range = true;
   static constexpr int cls = 2;
 };
+
+// Whether code on F takes the forms with fewer FP64 instructions.
+#ifdef TCG_PLAIN_FP64
+template <class F> constexpr bool SHORT64 = false;
+#else
+template <class F> constexpr bool SHORT64 = Prec<F>::cls == 0;
+#endif
 
 // Type of the literal constants in code on F (dual numbers take theirs as FP32 values,
 // which have no derivative to carry).
@@ -321,7 +335,7 @@ TCG_FN F xe_hot_of(const CellC<FC>& c, F lt, E&& ex = E()) {
   using K = typename ConstOf<F>::type;
   F eHe = ex(At<32>(), [&] { return (K(4.45) - lt) * K(1.0 / 0.06); });
   F xeHe;
-  if constexpr (Prec<F>::cls == 0) {  // one quotient (the product stays below 1e70)
+  if constexpr (SHORT64<F>) {  // one quotient (the product stays below 1e70)
     F a = K(1) + eHe, b = K(1) + eHe * K(4160.262005375057);
     xeHe = K(0.1) * (a + b) / over(a * b);
   } else {
@@ -477,12 +491,12 @@ TCG_FN void cool_terms(const CellC<FC>& c, const ChemT<F>& b, CoolT<F>& k, unsig
     k.rvLlow = ex(At<28>(), [&] { return poly * K(LN10); });
     F lT3 = lnTc - K(6.907755278982137);
     F iT3;  // 1/T3 = exp(-lT3)
-    if constexpr (Prec<F>::cls == 0) iT3 = K(1000) * m_min(m_max(invT, K(1e-4)), K(0.1));
+    if constexpr (SHORT64<F>) iT3 = K(1000) * m_min(m_max(invT, K(1e-4)), K(0.1));
     else iT3 = K(1000) / m_min(m_max(T, K(10)), K(1e4));
     k.rvLLTE = rovib_lte_of(lT3, iT3, ex);
   }
   F st10;
-  if constexpr (Prec<F>::cls == 0) st10 = b.sqT * K(0.31622776601683794);
+  if constexpr (SHORT64<F>) st10 = b.sqT * K(0.31622776601683794);
   else st10 = m_sqrt(T * K(0.1));
   k.coA = K(4e-27) * (T * K(0.1)) * st10;
   k.coN = K(3e3) * st10;
@@ -676,7 +690,7 @@ template <class F> TCG_BIG Equil<F> equilibrium(const CellC<F>& c, const ChemT<F
       if (dx <= tol * x || hi - lo <= tol * hi) break;
       // in FP64 a Newton step below 1e-8 of x has converged: what it leaves is about half its
       // square (g''/2g' x ~ 1/2), below rounding
-      if (Prec<F>::cls == 0 && newton && dx <= F(1e-8) * x) break;
+      if (SHORT64<F> && newton && dx <= F(1e-8) * x) break;
       // a caller whose guess is within ~1e-7 of the root (the Jacobian's perturbed
       // evaluations, started from the base point's root) stops after newton_max Newton
       // steps: one step from there is already converged to ~1e-14
@@ -735,7 +749,7 @@ template <class F> TCG_FN F dust_T(const CellC<F>& c, F T, F sqT, F guess) {
     F dy = m_abs(yn - y);
     y = yn;
     if (dy <= tol * y || hi - lo <= tol * hi) break;
-    if (Prec<F>::cls == 0 && newton && dy <= F(3e-9) * y) break;  // leaves ~5/2 of its square
+    if (SHORT64<F> && newton && dy <= F(3e-9) * y) break;  // leaves ~5/2 of its square
   }
   return y;
 }
