@@ -98,7 +98,7 @@ typedef struct tc_params {
                                   of a forward difference) and share FP64 exponentials (tc_step and
                                   tc_step_host only; other modes and tc_step_batch use 1).  0 (default): for TC_MODE_NEWTON_FP64 and
                                   TC_MODE_MIXED 4 on launches too small to fill the GPU, whose time is
-                                  the latency of the slowest cells (up to 64 and 32 cells per SM), else
+                                  the latency of the slowest cells (up to 64 and 128 cells per SM), else
                                   1, unless tc_autotune has recorded a choice for the launch's size class. */
 } tc_params;
 

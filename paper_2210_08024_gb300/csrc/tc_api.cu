@@ -307,21 +307,18 @@ static void default_block(int kmode, long long ntotal, int num_sms, int& b, int&
   }
 }
 
-// Whether a launch of modes 1 and 2 takes four lanes per cell: while the cells' warps of
-// eight are at most two (mode 1) or one (mode 2) per SM partition, where latency decides.  ms
-// with four / one: random states mode 1: 500 32 / 43, 4096 37 / 49, 8000 44 / 46; mode 2: 4096
-// 31 / 34, 8000 50 / 37; slab mode 1: 8000 4.5 / 5.4, mode 2: 8000 4.8 / 4.8; 12,800 curve
-// cells, mode 1: 24 / 15.
-static bool default_coop(int kmode, long long ntotal, int num_sms) {
-  return ntotal <= (long long)num_sms * 32 * ((kmode == 1) ? 2 : 1);
-}
-
-// The same for the drivers: four lanes while every cell's fit the resident lanes (19,456 cells).  A
-// cell's results on one and on four lanes differ by rounding (mode 1) or by the polish's
-// remainder (mode 2), which a driver's chunks can multiply (tc_k_driver.cuh), so this line lies
-// where it has always lain.
-static bool driver_coop(int kmode, long long ntotal, int num_sms) {
-  return ntotal * 4 <= (long long)num_sms * coop_occupancy(kmode, 128, true) * 128;
+// Whether a launch of modes 1 and 2 takes four lanes per cell.
+//  - Mode 1: while the cells' warps of eight are at most two per SM partition, where latency
+//    decides (four and one lane agree to 1e-13).  ms with four / one: random states: 500 32 / 43,
+//    4096 37 / 49, 8000 44 / 46; slab: 8000 4.5 / 5.4.
+//  - Mode 2, and mode 1 by the drivers: while every cell's lanes are resident at once (19,456
+//    cells).  One lane is faster from 4864 cells on (random states: 8000 50 / 37; slab: 8000 4.8 /
+//    4.8; curve cells, mode 1: 12,800 62 / 57), but its results differ: in mode 2 by the polish's
+//    remainder (x_CO by 1.5e-9 in 9 of 110 launches of random states, T by 6e-7 in one), in a
+//    driver by rounding that its chunks multiply (tc_k_driver.cuh).
+static bool default_coop(int kmode, long long ntotal, int num_sms, bool driver) {
+  if (kmode == 1 && !driver) return ntotal <= (long long)num_sms * 64;
+  return ntotal * 4 <= (long long)num_sms * coop_occupancy(kmode, 128, driver) * 128;
 }
 
 // Cells that a warp of the cooperative kernels advances at once: eight, or fewer where that
@@ -348,8 +345,7 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal,
   b = (b / 32) * 32;
   if (b < 32) b = 32;
   if (!coop_ok) lpc = 1;
-  if (lpc <= 0)
-    lpc = (coop_ok && (driver ? driver_coop(kmode, ntotal, h->num_sms) : default_coop(kmode, ntotal, h->num_sms))) ? 4 : 1;
+  if (lpc <= 0) lpc = (coop_ok && default_coop(kmode, ntotal, h->num_sms, driver)) ? 4 : 1;
   if (lpc != 4) lpc = 1;
   if (auto_block) {
     int ps = 0;
@@ -389,10 +385,13 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal,
 // over 100 yr 0.82 / 0.70, 4096 random states over 1e4 yr 36.2 / 30.9 (4800 over 100 yr 14.8 /
 // 16.2); mixed, 1500 slab cells over 1e4 yr 3.75 / 3.28, 4800 random states 32.3 / 33.9.  A cost
 // hint orders by the cost itself: alike cells then share a warp and its code (the PDR driver's
-// 48 x 100 cells 122 / 162 ms), so those and the drivers' first chunks stay with the queue.
-static int dealt_cells(const Shape& sh, long long ntotal) {
+// 48 x 100 cells 122 / 162 ms), so those and the drivers' first chunks stay with the queue, and so
+// do mixed launches of more than one warp per SM partition (16,000 cells, 1e4 yr: slab 4.96 / 7.02,
+// stiff 5.37 / 7.56, random states 65.5 / 72.8).
+static int dealt_cells(const Shape& sh, int kmode, long long ntotal, int num_sms) {
   const long long slots = (long long)sh.grid * sh.block / 32 * sh.groups;
-  return (sh.lpc == 4 && ntotal <= slots) ? (int)slots : 0;
+  const bool few = kmode == 1 || ntotal <= (long long)num_sms * 32;
+  return (sh.lpc == 4 && ntotal <= slots && few) ? (int)slots : 0;
 }
 
 // Grows the cost-ordering workspace to ncell cells (not while `st` is being captured).
@@ -441,7 +440,7 @@ static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long 
       return TC_ECUDA;
     h->launches += 3;
     dp.order = h->d_order;
-    if (!driver && !f.hint) dp.deal = dealt_cells(sh, ntotal);
+    if (!driver && !f.hint) dp.deal = dealt_cells(sh, kmode, ntotal, h->num_sms);
   }
   cudaError_t e;
   if (driver_kernel(kmode, driver)) {
