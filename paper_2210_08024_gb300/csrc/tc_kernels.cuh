@@ -337,7 +337,7 @@ TCG_FN bool solve3(F J[3][3], F b[3], F d[3]) {
       F tb = b[kk]; b[kk] = b[piv]; b[piv] = tb;
     }
     for (int i = kk + 1; i < 3; ++i) {
-      F m = J[i][kk] / J[kk][kk];
+      F m = J[i][kk] / over(J[kk][kk]);
       for (int j = kk; j < 3; ++j) J[i][j] -= m * J[kk][j];
       b[i] -= m * b[kk];
     }
@@ -345,7 +345,7 @@ TCG_FN bool solve3(F J[3][3], F b[3], F d[3]) {
   for (int i = 2; i >= 0; --i) {
     F acc = b[i];
     for (int j = i + 1; j < 3; ++j) acc -= J[i][j] * d[j];
-    d[i] = acc / J[i][i];
+    d[i] = acc / over(J[i][i]);
   }
   return true;
 }
@@ -593,15 +593,16 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 //     step each), until a step is below 3e-5 or stops shrinking at FP32's rounding floor.
 //     This takes the varying part of the iteration counts, which would leave lanes of a
 //     warp waiting, off the FP64 pipe.
-//  2. FP64: f in FP64 at the FP32 root (~1e-6 off), the correction with the FP32 Jacobian of
-//     the last dual-number evaluation (rebuilt at the iterate when a step does not shrink a
-//     thousandfold).  Two evaluations usually do.
-// Converged when every step is below rtol |y_i| as in newton_iter, or one step earlier,
-// when two steps in a row show that the next would lie far below it: with rho = d_k /
-// d_(k-1), what remains after step k is at most ~rho d_k, accepted below 1e-2 rtol.  The C/O/e
-// equilibrium of the last evaluation is moved along the last step by its derivatives.  2-norm
-// errors on 20,000 slab cells against roots solved to rounding: T 1.1e-16, x_e 1.8e-16; by the
-// plain iteration 3.9e-15, 4.7e-14.
+//  2. FP64: f in FP64 at the FP32 root (~1e-6 off), the correction by an FP64 solve with the FP32
+//     Jacobian of the last dual-number evaluation.  Rebuilt at the iterate when a step does not
+//     shrink a thousandfold, or moved an abundance by more than 1% (TAN_STALE: the derivatives of
+//     its rate are proportional to it).  Two evaluations usually do.
+// Converged when every step is below rtol of its unknown, or when what remains is below 1e-2
+// rtol: after step k about rho d_k, with rho = d_k / d_(k-1), and after the first step at most d_1
+// times the error of its Jacobian.  The C/O/e equilibrium of the last evaluation is moved along
+// the last step by its derivatives.  2-norm errors on 20,000 slab cells against roots solved to
+// rounding: T 1.1e-16, x_e 1.8e-16; by the plain iteration 3.9e-15, 4.7e-14.  Largest errors of
+// x_H2 down to 1e-20 (20,000 stiff cells, 4096 random states): 9e-13, 2e-13; plain 1e-13, 2e-13.
 //
 // Returns the iterations of both phases, or -1 when a step would have to be damped, fails to
 // shrink by half or is not finite, or when TAN_MAXIT iterations pass; the plain solver then
@@ -612,6 +613,7 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 // x_H = 0.)
 constexpr int TAN_MAXIT = 12;
 constexpr int TAN_MAXIT32 = 16;
+constexpr float TAN_STALE = 1e-2f;  // a Jacobian whose abundances were further off is rebuilt
 constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
 
 // source_tangents over the cell's lanes: with four, each takes one direction (the last
@@ -655,6 +657,7 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
   const float h = float(dts);
   float df[3][3], dq[3][3], dtd[3];
   int it32 = 0, res = -1;
+  bool fresh = false;  // rebuild the Jacobian at the next iterate
   // Both loops leave through their one end, with a flag, so that the lanes of a warp meet
   // again there: a return inside let each exit run the second phase on its own.
   bool ok = true;
@@ -710,6 +713,7 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       td = v.td + v.dtd[0] * u[0] + v.dtd[1] * u[1] + v.dtd[2] * u[2];
 #pragma unroll
       for (int i = 0; i < 3; ++i) dtd[i] = v.dtd[i];
+      fresh = fabsf(u[1]) > TAN_STALE * x[1] || fabsf(u[2]) > TAN_STALE * x[2];
       if (whole && rel < 3e-5f) break;
       if (whole && !(rel <= 0.5f * prev) && it32 > 2) {
         ok = rel < 1e-3f;  // FP32's rounding floor
@@ -730,7 +734,6 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
   }
   // ---- phase 2
   float prev = -1.0f;  // size of the previous step, if that was whole
-  bool fresh = false;  // rebuild the Jacobian at the next iterate
   for (int it = 1; ok && it <= TAN_MAXIT; ++it) {
     TCG_COUNT_D(tangent_it);
     double f[3];
@@ -743,41 +746,29 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
     const double xH = 1.0 - 2.0 * y[1] - y[2];
     const float y0 = float(y[0]), x2 = float(y[1]), xp = float(y[2]);
     if (fresh) tangents<LPC>(cf, p.flags, hk, float(mu) * y0, x2, xp, float(xH), float(xe_g), float(td_g), df, dq);
-    // rows scaled: (T_mu equation / T_mu, x_H2, x_H+); unknowns (ln T_mu, x_H2, x_H+)
+    // rows scaled: (T_mu equation / T_mu, x_H2, x_H+); unknowns (ln T_mu, x_H2, x_H+).  The
+    // Jacobian is FP32's, its solution FP64's: in hot ionised gas the step of x_H2 is a small
+    // difference of terms of x_H+, which FP32 loses, and with it the sight of an x_H2 that has
+    // not converged (x_H2 = 1e-20 to 1e-15 was off by up to 2e-2 of itself).
     const float iy0 = 1.0f / y0;
-    float J[3][3], r[3], u[3];
-    double d[3], rhs[3];
+    double J[3][3], r[3], d[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      rhs[i] = -(y[i] - yn[i] - dts * f[i]);
       const float s = (i == 0) ? iy0 : 1.0f;
-      r[i] = float(rhs[i]) * s;
+      r[i] = -(y[i] - yn[i] - dts * f[i]) * double(s);
 #pragma unroll
-      for (int j = 0; j < 3; ++j) J[i][j] = ((i == j) ? 1.0f : 0.0f) - (h * s) * df[i][j];
-      // an abundance near or below FP32's range matters to nothing but itself: its row
-      // decouples and its step is taken in FP64
-      if (i > 0 && y[i] < TAN_TRACE) {
-        d[i] = rhs[i] / double(J[i][i]);
-        r[i] = 0.0f;
-        J[i][0] = J[i][3 - i] = 0.0f;
-      }
+      for (int j = 0; j < 3; ++j) J[i][j] = double(((i == j) ? 1.0f : 0.0f) - (h * s) * df[i][j]);
     }
-    // what one rounding of the other unknowns moves an abundance by
-    const float eps = 1.2e-16f;
-    const float noise[3] = {0.0f, eps * (fabsf(J[1][0]) + fabsf(J[1][2]) * xp) / fabsf(J[1][1]),
-                            eps * (fabsf(J[2][0]) + fabsf(J[2][1]) * x2) / fabsf(J[2][2])};
-    ok = solve3<float>(J, r, u);
+    ok = solve3<double>(J, r, d);
+    const float u[3] = {float(d[0]), float(d[1]), float(d[2])};
     // T_mu, x_H2, x_H+ and x_H must keep 2% of their values (damped_step limits at 1%),
     // except an abundance whose step is below 1e-8 (too little to matter to the others): it
     // may fall to any positive value, and to 1% of its value where the step rounds to less
     bool whole = true;
     float rel = fabsf(u[0]);
-    d[0] = double(u[0]) * y[0];
+    d[0] *= y[0];
 #pragma unroll
     for (int i = 1; i < 3; ++i) {
-      const bool trace = y[i] < TAN_TRACE;
-      if (trace) u[i] = float(d[i]);
-      else d[i] = double(u[i]);
       const float x = (i == 1) ? x2 : xp;
       if (fabsf(u[i]) <= 1e-8f) {
         if (!(y[i] + d[i] > 0.0) && d[i] != 0.0) {
@@ -787,17 +778,15 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       } else {
         ok = ok && u[i] >= -0.98f * x;
       }
-      const double yi = y[i] + d[i];
-      const float ri = trace ? float(fabs(d[i]) / (fabs(yi) + 1e-300)) : fabsf(u[i]) / (fabsf(float(yi)) + 1e-30f);
-      // (in hot gas the rounding of x_H = 1 - 2 x_H2 - x_H+ moves x_H2 by up to 1e-5 of itself,
-      // back and forth: such a step is no distance from the root)
-      if (!(fabsf(u[i]) <= noise[i])) rel = fmaxf(rel, ri);
+      const double yi = fabs(y[i] + d[i]);
+      rel = fmaxf(rel, (y[i] < TAN_TRACE) ? float(fabs(d[i]) / (yi + 1e-300)) : fabsf(u[i]) / (float(yi) + 1e-30f));
     }
     ok = ok && u[0] >= -0.98f && -2.0f * u[1] - u[2] >= -0.98f * float(xH) && isfinite(rel);
     if (!ok) break;
     y[0] += d[0]; y[1] += d[1]; y[2] += d[2];
     if (!whole) {
       prev = -1.0f;
+      fresh = true;
       continue;
     }
     const double dxe = double(dq[0][0] * u[0] + dq[0][1] * u[1] + dq[0][2] * u[2]);
@@ -825,7 +814,7 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
       break;
     }
     if (it > 2 && prev > 0.0f && !(rel <= 0.5f * prev)) break;
-    fresh = prev > 0.0f && rel > 1e-3f * prev;
+    fresh = (prev > 0.0f && rel > 1e-3f * prev) || rel > TAN_STALE;
     prev = rel;
     // the next evaluation's inner roots, predicted along the step
     xe_g += dxe;
