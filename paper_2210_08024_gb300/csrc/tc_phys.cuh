@@ -170,6 +170,10 @@ template <class F> constexpr bool SHORT64 = Prec<F>::cls == 0;
 // which have no derivative to carry).
 template <class F> struct ConstOf { using type = F; };
 
+// Rates at or below this are taken as none: 0, and for dual numbers FP32's smallest normal values,
+// whose approximate reciprocal would be infinite (H2's ro-vibrational cooling below 15 K).
+template <class F> constexpr double LEAST_RATE = (Prec<F>::cls == 3) ? 2e-38 : 0.0;
+
 // A value computed at run time, in precision F (df64 keeps subnormal trailing parts on
 // the device; constants convert at compile time with F(x)).
 template <class F> TCG_FN F to_prec(double x) { return F(x); }
@@ -838,7 +842,7 @@ template <class F, class FC> TCG_BIG Src<F> source(const CellC<FC>& c, const Che
     F Lrv;
     if constexpr (Prec<F>::fp32_range) Lrv = k.rvLLTE * (nL / den);
     else Lrv = k.rvLLTE * nL / over(den);
-    Lhyd += (den > K(0)) ? xH2 * Lrv / over(n) : K(0);
+    Lhyd += (den > K(LEAST_RATE<F>)) ? xH2 * Lrv / over(n) : K(0);
   }
   F Lmet;
   {
