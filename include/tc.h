@@ -76,7 +76,9 @@ typedef struct tc_params {
   double fd_rel_step;          /* relative FD step for dH/dT_mu (mode 0); default 1e-3 */
   double newton_rtol;          /* Newton tolerance, FP64 modes; default 1e-12 */
   double T_floor;              /* temperature floor [K]; default 1 */
-  int newton_max;              /* Newton iteration cap; default 50 */
+  int newton_max;              /* Newton iteration cap of a solve, FP32 iterations included; default 50.
+                                  (TC_MODE_NEWTON_FP64 below 28: the plain FP64 iteration alone, whose
+                                  restarts and halvings depend on it) */
   int max_substeps;            /* substep cap per cell; default 1e6 */
   int mode;                    /* TC_MODE_* */
   unsigned flags;              /* TC_CONST_KGR | TC_NO_ROVIB | TC_NO_CIE */

@@ -1077,7 +1077,7 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
       s.status |= ST_SEED_FAIL;
     }
   }
-  if (src) {
+  if (src && p.newton_max >= TAN_MAXIT32 + TAN_MAXIT) {  // a tighter cap is the plain iteration's to keep
     double xg = xe_g, tg = td_g;
     it = newton_tangent<LPC>(c, *cf, p, s.mu, Kinv, yn, dts, y, xg, tg, &qb);
     if (it >= 0) { xe_g = xg; td_g = tg; }
