@@ -108,13 +108,14 @@ TCG_FN double m_abs(double a) { return fabs(a); }
 TCG_FN float m_abs(float a) { return fabsf(a); }
 
 // Quotients of the FP64 physics on the device: the approximate reciprocal (MUFU, ~2^-20), one
-// third-order step and one residual correction, 6 FP64 instructions and no slow path; error
-// below 0.51 ulp (tests/test_gpu_div64.py).  Exponents from which a step could leave the range
-// take the plain division.
+// third-order step and the residual correction of Markstein (IBM J. Res. Dev. 34, 111, 1990), 6
+// FP64 instructions and no slow path; error below 0.51 ulp (tests/test_gpu_div64.py), below one
+// unit where the quotient is subnormal.  Taken for |b| in [2^-511, 2^513) and |a| < 2^512, so that
+// the quotient stays below 2^1023 and every step in range; other operands take the plain division.
 TCG_FN double m_div(double a, double b) {
 #if defined(__CUDA_ARCH__) && !defined(TCG_PLAIN_FP64)
-  if ((unsigned)((hi_word(b) & 0x7fffffff) - 0x10000000) < 0x60000000u &&
-      (unsigned)(hi_word(a) & 0x7fffffff) < 0x70000000u) {
+  if ((unsigned)((hi_word(b) & 0x7fffffff) - 0x20000000) < 0x40000000u &&
+      (unsigned)(hi_word(a) & 0x7fffffff) < 0x5ff00000u) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
     const double e = fma(-b, y, 1.0);
