@@ -108,7 +108,7 @@ __device__ __forceinline__ void weights(double x, double& p, double& q) {
   const int m = e >> 9;
   p = fma(y, y, 2.0 * (y * lo));
   q = fma(p, y, p * lo);
-  if (x < -236.0) {  // a product may leave the normal range
+  if (!(x >= -236.0)) {  // a product may leave the normal range; NaN, whose bits are no exponent's
     const double h = exp64(x);
     p = h * h;
     q = p * h;
