@@ -122,8 +122,9 @@ typedef struct tc_fields {
   long long ncell;
   double Zg_val, Zd_val;    /* scalars used when Zg / Zd are NULL */
   int *newton_iters;        /* optional out (device, may be NULL): Newton iterations summed over the
-                               cell's substeps (modes 1-4; the mixed modes count FP32 iterations;
-                               the seeded modes include abandoned seeded attempts) */
+                               cell's substeps (modes 1-4; TC_MODE_NEWTON_FP64 counts the FP32 and
+                               FP64 iterations of its two phases, the mixed modes FP32 ones;
+                               abandoned attempts, seeded or not, are included) */
   const int *cost_hint;     /* optional in (device, may be NULL; tc_step and tc_step_batch only): a
                                per-cell cost estimate, larger = costlier, for example the newton_iters
                                output of the cell's previous step.  With tc_params.order_cells set,

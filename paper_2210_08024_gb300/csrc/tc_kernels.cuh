@@ -604,7 +604,7 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 // rounding: T 1.1e-16, x_e 1.8e-16; by the plain iteration 3.9e-15, 4.7e-14.  Largest errors of
 // x_H2 down to 1e-20 (20,000 stiff cells, 4096 random states): 9e-13, 2e-13; plain 1e-13, 2e-13.
 //
-// Returns the iterations of both phases, or -1 when a step would have to be damped, fails to
+// `spent` receives the iterations of both phases.  Returns them, or -1 when a step would have to be damped, fails to
 // shrink by half or is not finite, or when TAN_MAXIT iterations pass; the plain solver then
 // takes the substep from its start, as if this one had not been tried.  Hard substeps (2% of
 // the random states' iterations, 0.04% of the slab's) thus keep the plain iteration's path,
@@ -652,7 +652,8 @@ TCG_FN void tangents(const CellC<float>& c, unsigned flags, float hk, float T, f
 
 template <int LPC = 1>
 TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double mu, double Kinv,
-                          const double* yn, double dts, double* y, double& xe_g, double& td_g, Equil<double>* qb) {
+                          const double* yn, double dts, double* y, double& xe_g, double& td_g, Equil<double>* qb,
+                          int* spent) {
   const float hk = float(1.0 / (double(c.muH) * KB * 1.5));
   const float h = float(dts);
   float df[3][3], dq[3][3], dtd[3];
@@ -734,8 +735,10 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
   }
   // ---- phase 2
   float prev = -1.0f;  // size of the previous step, if that was whole
+  int it64 = 0;
   for (int it = 1; ok && it <= TAN_MAXIT; ++it) {
     TCG_COUNT_D(tangent_it);
+    it64 = it;
     double f[3];
     {
       ChemT<double> b;
@@ -820,6 +823,7 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
     xe_g += dxe;
     td_g += double(dtd[0] * u[0] + dtd[1] * u[1] + dtd[2] * u[2]);
   }
+  *spent = it32 + it64;
   return res;
 }
 
@@ -1050,13 +1054,13 @@ TCG_FN int chord64_from_seed(const CellC<double>& c, const CellC<float>& cf, con
 
 // Solves one substep of length dts by the FP64 Newton iteration, from `seed` when
 // given (the root is the same; a seeded solve that fails is retried from the start
-// state), else from the start state (with `src`, the start's source terms, first by
-// newton_tangent), then from the predictor; a substep that fails from both is retried
+// state), else from the start state (with `tangent`, first by newton_tangent, which takes the
+// FP32 constants cf), then from the predictor; a substep that fails from both is retried
 // at half length (up to 30 times) and the cell flagged ST_NEWTON.
 template <int LPC = 1>
 TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double dt, double dts, bool last,
                             LaneState& s, double& xe_g, double& td_g, const double* seed = nullptr,
-                            const CellC<float>* cf = nullptr, const double* src = nullptr) {
+                            const CellC<float>* cf = nullptr, bool tangent = false) {
   const double yn[3] = {s.Tmu, s.xH2, s.xHp};
   const double Kinv = 1.0 / c.K;
   double y[3] = {yn[0], yn[1], yn[2]};
@@ -1077,10 +1081,15 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
       s.status |= ST_SEED_FAIL;
     }
   }
-  if (src && p.newton_max >= TAN_MAXIT32 + TAN_MAXIT) {  // a tighter cap is the plain iteration's to keep
+  if (tangent && p.newton_max >= TAN_MAXIT32 + TAN_MAXIT) {  // a tighter cap is the plain iteration's to keep
     double xg = xe_g, tg = td_g;
-    it = newton_tangent<LPC>(c, *cf, p, s.mu, Kinv, yn, dts, y, xg, tg, &qb);
-    if (it >= 0) { xe_g = xg; td_g = tg; }
+    int spent = 0;
+    it = newton_tangent<LPC>(c, *cf, p, s.mu, Kinv, yn, dts, y, xg, tg, &qb, &spent);
+    if (it >= 0) {
+      xe_g = xg; td_g = tg;
+    } else {
+      s.iters += spent;   // the abandoned iterations count here as well
+    }
   }
   if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);
   int halv = 0;
@@ -1122,13 +1131,13 @@ template <int LPC = 1>
 TCG_FN void substep_newton64(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double dt, LaneState& s,
                              double& xe_g, double& td_g) {
   bool last;
-  double src[3];
-  const double dts = substep_start64<LPC>(c, p, dt, s, td_g, last, src);
+  const double dts = substep_start64<LPC>(c, p, dt, s, td_g, last);
 #ifdef TCG_DRIVER
-  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g);  // by the plain iteration
+  constexpr bool tangent = false;
 #else
-  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, src);
+  constexpr bool tangent = true;
 #endif
+  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, tangent);
 }
 template <int LPC = 1>
 TCG_FN void substep_newton64(const CellC<double>& c, const DevParams& p, double dt, LaneState& s, double& xe_g,

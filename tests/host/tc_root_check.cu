@@ -5,8 +5,9 @@
 // Usage: tc_root_check IN
 //   IN: n as int64, then 12 arrays of n doubles (n, chi_pe, chi_lw, f_shld_H2, f_shld_C,
 //       F_LyC, xi, Z'_g, Z'_d, T, x_H2, x_H+), then dt as a double.
-// Prints one JSON object: substeps, those that newton_tangent left to the plain iteration, those
-// without a long double root, and the largest relative error of T_mu, x_H2 and x_H+ (the abundances where above 1e-20) after it.
+// Prints one JSON object: substeps, those that newton_tangent left to the plain iteration (and
+// of these, those that do not count its iterations), those without a long double root, and the
+// largest relative error of T_mu, x_H2 and x_H+ (the abundances where above 1e-20) after it.
 #include <math.h>
 
 // long double forms of the functions the physics templates call (declared ahead of them)
@@ -95,7 +96,7 @@ int main(int argc, char** argv) {
   f.n = col(0); f.chi_pe = col(1); f.chi_lw = col(2); f.fh2 = col(3); f.fc = col(4);
   f.Flyc = col(5); f.xi = col(6); f.Zg = col(7); f.Zd = col(8);
   f.T = col(9); f.xH2 = col(10); f.xHp = col(11);
-  long long nsub = 0, left = 0, noroot = 0;
+  long long nsub = 0, left = 0, miscounted = 0, noroot = 0;
   double worst[3] = {0, 0, 0};
   for (int64_t i = 0; i < n; ++i) {
     CellC<double> c;
@@ -116,9 +117,15 @@ int main(int argc, char** argv) {
       const double yn[3] = {s.Tmu, s.xH2, s.xHp};
       double y[3] = {yn[0], yn[1], yn[2]}, xg = xe_g, tg = td_g;
       Equil<double> q;
+      int spent = 0;
       ++nsub;
-      if (newton_tangent<1>(c, cf, p, s.mu, 1.0 / c.K, yn, dts, y, xg, tg, &q) < 0) {
+      if (newton_tangent<1>(c, cf, p, s.mu, 1.0 / c.K, yn, dts, y, xg, tg, &q, &spent) < 0) {
         ++left;
+        LaneState a = s, b = s;  // with the abandoned iterations, and by the plain iteration alone
+        double xa = xe_g, ta = td_g, xb = xe_g, tb = td_g;
+        solve_substep64<1>(c, p, dt, dts, last, a, xa, ta, nullptr, &cf, true);
+        solve_substep64<1>(c, p, dt, dts, last, b, xb, tb);
+        if (a.iters != b.iters + spent || a.Tmu != b.Tmu) ++miscounted;
       } else {
         Problem P{cast_cell<LD>(c), p.flags, s.mu, 1 / LD(c.K), dts, {yn[0], yn[1], yn[2]}};
         LD z[3] = {y[0], y[1], y[2]};
@@ -132,10 +139,10 @@ int main(int argc, char** argv) {
           }
         }
       }
-      solve_substep64<1>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, worst);
+      solve_substep64<1>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, true);
     }
   }
-  printf("{\"substeps\": %lld, \"left\": %lld, \"noroot\": %lld, \"T\": %.3e, \"xH2\": %.3e, \"xHp\": %.3e}\n", nsub, left,
-         noroot, worst[0], worst[1], worst[2]);
+  printf("{\"substeps\": %lld, \"left\": %lld, \"miscounted\": %lld, \"noroot\": %lld, \"T\": %.3e, \"xH2\": %.3e, \"xHp\": %.3e}\n", nsub,
+         left, miscounted, noroot, worst[0], worst[1], worst[2]);
   return 0;
 }

@@ -63,5 +63,6 @@ def test_roots_match_long_double(check, tmp_path, workload, dt_yr):
             fh.write(np.ascontiguousarray(np.broadcast_to(np.asarray(v, np.float64), (n,))).tobytes())
         fh.write(np.float64(dt_yr * 3.15576e7).tobytes())
     r = json.loads(subprocess.run([check, str(path)], check=True, capture_output=True, text=True).stdout)
+    assert r["miscounted"] == 0, r  # an abandoned solve's iterations are in newton_iters
     assert r["noroot"] == 0 and r["left"] < 0.02 * r["substeps"], r
     assert max(r[k] for k in ("T", "xH2", "xHp")) <= 2e-12, r
