@@ -350,6 +350,9 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal,
   if (auto_block) {
     int ps = 0;
     default_block(kmode, ntotal, h->num_sms, b, ps);
+    // the drivers' plain iteration fills more warps (512,000 curve cells, ms at 2 / 4 blocks per
+    // SM / the limit: 537 / 526 / 523; 300,000 slab cells 1262 / 1576 / 1906)
+    if (driver_kernel(kmode, driver) && b == 128 && ps == 2) ps = 4;
     if (lpc == 4) {
       if (b > tcg::STEP_THREADS) b = tcg::STEP_THREADS;
     } else if (per_sm <= 0) {

@@ -145,6 +145,12 @@ TCG_FN void temp_blocks(const CellC<FC>& c, F T, unsigned flags, bool eq, ChemT<
   k = cool_T(c, b, flags);
 }
 
+// The FP64 temperature blocks at a substep's start, where they are kept.
+struct TempBlocks {
+  ChemT<double> b;
+  CoolT<double> k;
+};
+
 // Work-queue claim for cells of LPC lanes: the first lane of the cell takes the next
 // index and hands it to the others by a shuffle over the cell's explicit lane mask
 // (__activemask could return part of a cell whose lanes are briefly apart, so the
@@ -433,7 +439,7 @@ constexpr double JAC_REUSE = 1e-3;
 template <int LPC = 1>
 TCG_FN int newton_iter(const CellC<double>& c, const DevParams& p, double mu, double Kinv, const double* yn,
                        double dts, double* y, double& xe_g, double& td_g, double (*Jk)[3], bool reuse,
-                       double& rel, bool& full, Equil<double>* qb) {
+                       double& rel, bool& full, Equil<double>* qb, const TempBlocks* tb = nullptr) {
   double f0[3], J[3][3];
   if constexpr (LPC == 4) {
     if (reuse) {
@@ -486,11 +492,20 @@ TCG_FN int newton_iter(const CellC<double>& c, const DevParams& p, double mu, do
     // then the T_mu column from the base point's temperature blocks stepped to T + dT
     // (temp_blocks_step).  The columns start their C/O/e and dust-temperature solves from the base
     // point's roots, ~1e-7 away, and take one Newton step of the C/O/e balance
-    // (converged to ~1e-14 from there; the loop would take a second to confirm it).
+    // (converged to ~1e-14 from there; the loop would take a second to confirm it).  The
+    // temperature blocks at the base point are given by the caller at a substep's first
+    // iteration (the substep start's, the same temperature), else built here.
     if (reuse) TCG_COUNT_D(chord64_it);
     else TCG_COUNT_D(newton64_it);
-    ChemT<double> b = chem_T(c, mu * y[0], p.flags);
-    CoolT<double> k = cool_T(c, b, p.flags);
+    ChemT<double> b;
+    CoolT<double> k;
+    if (tb) {
+      b = tb->b;
+      k = tb->k;
+    } else {
+      b = chem_T(c, mu * y[0], p.flags);
+      k = cool_T(c, b, p.flags);
+    }
     feval64(c, b, k, y[1], y[2], Kinv, xe_g, td_g, f0, qb);
     if (reuse) {
       for (int i = 0; i < 3; ++i)
@@ -544,7 +559,7 @@ TCG_FN int newton_iter(const CellC<double>& c, const DevParams& p, double mu, do
 template <int LPC = 1>
 TCG_FN int newton_solve(const CellC<double>& c, const DevParams& p, double mu, double Kinv, const double* yn,
                         double dts, double* y, double& xe_g, double& td_g, int maxit = 0,
-                        Equil<double>* qb = nullptr, int* spent = nullptr) {
+                        Equil<double>* qb = nullptr, int* spent = nullptr, const TempBlocks* tb = nullptr) {
   const int nmax = (maxit > 0) ? maxit : p.newton_max;
   double Jk[3][3];
   bool reuse = false;
@@ -552,7 +567,8 @@ TCG_FN int newton_solve(const CellC<double>& c, const DevParams& p, double mu, d
   for (int it = 1; it <= nmax; ++it) {
     double rel;
     bool full;
-    const int r = newton_iter<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, Jk, reuse, rel, full, qb);
+    const int r = newton_iter<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, Jk, reuse, rel, full, qb,
+                                   (it == 1) ? tb : nullptr);
     if (spent) *spent = it;
     if (r < 0) return -1;
     if (r > 0) return it;
@@ -566,11 +582,17 @@ TCG_FN int newton_solve(const CellC<double>& c, const DevParams& p, double mu, d
 // with the dust temperature solved; gives the substep length of Sec. 6.1.
 template <class F, int LPC = 1>
 TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneState& s, F& td_g, double& H0,
-                          double& CH2, double& CHp) {
+                          double& CH2, double& CHp, TempBlocks* tb = nullptr) {
   const double T = s.mu * s.Tmu;
   ChemT<F> b;
   CoolT<F> k;
-  temp_blocks<LPC>(cf, to_prec<F>(T), p.flags, false, b, k);
+  temp_blocks<LPC>(cf, to_prec<F>(T), p.flags, tb != nullptr, b, k);
+  if constexpr (std::is_same_v<F, double>) {
+    if (tb) {
+      tb->b = b;
+      tb->k = k;
+    }
+  }
   Equil<F> q;
   q.xe = to_prec<F>(s.xe); q.xCp = to_prec<F>(s.xCp); q.xCO = to_prec<F>(s.xCO);
   q.xOp = cf.xOtot * to_prec<F>(s.xHp);
@@ -927,9 +949,10 @@ constexpr int RESCUE_ITER_FACTOR = 8;
 // solve, or -1.
 template <int LPC = 1>
 TCG_FN int solve_from_start64(const CellC<double>& c, const DevParams& p, double mu, double Kinv, const double* yn,
-                              double dts, double* y, double& xe_g, double& td_g, int& status, Equil<double>* qb) {
+                              double dts, double* y, double& xe_g, double& td_g, int& status, Equil<double>* qb,
+                              const TempBlocks* tb = nullptr) {
   y[0] = yn[0]; y[1] = yn[1]; y[2] = yn[2];
-  int it = newton_solve<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, 0, qb);
+  int it = newton_solve<LPC>(c, p, mu, Kinv, yn, dts, y, xe_g, td_g, 0, qb, nullptr, tb);
   if (it >= 0) return it;
   status |= ST_PREDICTOR;
   picard_predictor(c, p, mu, Kinv, yn, dts, y, xe_g, td_g);
@@ -1060,7 +1083,8 @@ TCG_FN int chord64_from_seed(const CellC<double>& c, const CellC<float>& cf, con
 template <int LPC = 1>
 TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double dt, double dts, bool last,
                             LaneState& s, double& xe_g, double& td_g, const double* seed = nullptr,
-                            const CellC<float>* cf = nullptr, bool tangent = false) {
+                            const CellC<float>* cf = nullptr, bool tangent = false,
+                            const TempBlocks* tb = nullptr) {
   const double yn[3] = {s.Tmu, s.xH2, s.xHp};
   const double Kinv = 1.0 / c.K;
   double y[3] = {yn[0], yn[1], yn[2]};
@@ -1091,14 +1115,14 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
       s.iters += spent;   // the abandoned iterations count here as well
     }
   }
-  if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);
+  if (it < 0) it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb, tb);
   int halv = 0;
   while (it < 0 && halv < 30) {
     s.status |= ST_NEWTON;
     dts *= 0.5;
     last = false;
     ++halv;
-    it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb);
+    it = solve_from_start64<LPC>(c, p, s.mu, Kinv, yn, dts, y, xe_g, td_g, s.status, &qb, tb);
   }
   if (it < 0) {
     s.status |= ST_NONFIN;
@@ -1114,16 +1138,16 @@ TCG_FN void solve_substep64(const CellC<double>& c, const DevParams& p, double d
 // factor.  `src`, when given, receives those terms (H, C_H2, C_H+).
 template <class F, int LPC = 1>
 TCG_FN double substep_start_t(const CellC<F>& cc, double K, const DevParams& p, double dt, const LaneState& s,
-                              F& td_g, bool& last, double* src = nullptr) {
+                              F& td_g, bool& last, double* src = nullptr, TempBlocks* tb = nullptr) {
   double H0, CH2, CHp;
-  start_sources<F, LPC>(cc, p, s, td_g, H0, CH2, CHp);
+  start_sources<F, LPC>(cc, p, s, td_g, H0, CH2, CHp, tb);
   if (src) { src[0] = H0; src[1] = CH2; src[2] = CHp; }
   return substep_len(p, dt - s.t, K * s.Tmu, H0, CH2, CHp, last);
 }
 template <int LPC = 1>
 TCG_FN double substep_start64(const CellC<double>& c, const DevParams& p, double dt, const LaneState& s,
-                              double& td_g, bool& last, double* src = nullptr) {
-  return substep_start_t<double, LPC>(c, c.K, p, dt, s, td_g, last, src);
+                              double& td_g, bool& last, double* src = nullptr, TempBlocks* tb = nullptr) {
+  return substep_start_t<double, LPC>(c, c.K, p, dt, s, td_g, last, src, tb);
 }
 
 // One substep of mode 1; cf is the FP32 copy of the cell's constants.
@@ -1131,13 +1155,17 @@ template <int LPC = 1>
 TCG_FN void substep_newton64(const CellC<double>& c, const CellC<float>& cf, const DevParams& p, double dt, LaneState& s,
                              double& xe_g, double& td_g) {
   bool last;
-  const double dts = substep_start64<LPC>(c, p, dt, s, td_g, last);
 #ifdef TCG_DRIVER
-  constexpr bool tangent = false;
+  // by the plain iteration; with one lane per cell the start's temperature blocks serve its first
+  // evaluation (512,000 curve cells over 10 chunks 551 -> 523 ms)
+  TempBlocks tb;
+  TempBlocks* const t = (LPC == 1) ? &tb : nullptr;
+  const double dts = substep_start64<LPC>(c, p, dt, s, td_g, last, nullptr, t);
+  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, nullptr, false, t);
 #else
-  constexpr bool tangent = true;
+  const double dts = substep_start64<LPC>(c, p, dt, s, td_g, last);
+  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, true);
 #endif
-  solve_substep64<LPC>(c, p, dt, dts, last, s, xe_g, td_g, nullptr, &cf, tangent);
 }
 template <int LPC = 1>
 TCG_FN void substep_newton64(const CellC<double>& c, const DevParams& p, double dt, LaneState& s, double& xe_g,
