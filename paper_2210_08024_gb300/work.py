@@ -12,8 +12,8 @@ scalar type; its counts per iteration are stated here from the code:
     FP64 Newton iteration   63 add, 55 mul, 16 div   (one division per Jacobian column)
     FP64 chord iteration    42 add, 40 mul, 13 div   (the same without the differencing:
                                                       21 add, 15 mul, 9 div)
-    dual-number iteration   11 add,  6 mul           (its FP64 part: residual and step; the
-                                                      Jacobian and the correction are FP32)
+    dual-number iteration   25 add, 21 mul,  6 div   (its FP64 part: residual, 3x3 solve and
+                                                      step; the Jacobian is FP32)
     mixed Newton iteration  18 add, 12 mul,  6 div   (its FP64 part: residual, damped step
                                                       and test; the correction is solved in FP32)
     polish iteration        16 add, 12 mul,  6 div   (the same, residual from df64 sources)
@@ -49,7 +49,7 @@ OUT = os.path.join(HERE, "work_slab128.json")
 LINALG = {
     "newton64_it": {"add": 63, "mul": 55, "div": 16},
     "chord64_it": {"add": 42, "mul": 40, "div": 13},
-    "tangent_it": {"add": 11, "mul": 6, "div": 0},
+    "tangent_it": {"add": 25, "mul": 21, "div": 6},
     "newton32_it": {"add": 18, "mul": 12, "div": 6},
     "polish_it": {"add": 16, "mul": 12, "div": 6},
     "substep_paper": {"add": 18, "mul": 18, "div": 8},
