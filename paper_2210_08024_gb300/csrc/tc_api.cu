@@ -291,14 +291,23 @@ struct Shape {
 //    14.8 / 11.8 / 10.5 / 10.5, 2M 44.4 (128) / 36.2 / 33.5; random states: 4k 40 / 44 / 50 / 62, 30k
 //    76 / 58 / 59 / 69, 100k 178 / 155 / 114 / 98.  At 100k one block of 256 an SM instead of
 //    the limit: slab seeded 7.2 -> 6.7, random states mixed 74 -> 62.
-static void default_block(int kmode, long long ntotal, int num_sms, int& b, int& per_sm) {
+//    Over short steps most cells take one substep, and seeded blocks of 256 mostly wait for the
+//    few that take more (ms with 256 (one an SM) / 128 / before the blocks met: stiff cells 100k
+//    over 100 yr 3.7 / 3.2 / 3.1, 300 yr 4.7 / 3.7 / 3.7, 1e3 yr 4.8 / 4.9 / 5.1; 160k over 100 yr
+//    4.2 / 3.9 / 3.9, 300 yr 4.7 / 4.5 / 4.9; slab cells over 100 yr, 170k 1.67 / 1.48 / 1.63).
+//    (Random states pay for it: 100k over 100 yr 40 / 64 / 95.)
+constexpr double SHORT_STEP = 500.0 * 3.15576e7;
+static void default_block(int kmode, long long ntotal, int num_sms, double dt, int& b, int& per_sm) {
   const long long per = ntotal / num_sms;
   per_sm = 0;
   if (per < 112) {
     b = 32;
   } else if (kmode == 2 || kmode == 3) {
     b = (per < 600) ? 128 : (per < 1600) ? 256 : 512;
-    if (b == 256 && per < 1200) per_sm = 1;
+    if (b == 256 && per < 1200) {
+      if (kmode == 3 && dt < SHORT_STEP) b = 128;
+      else per_sm = 1;
+    }
   } else {
     b = (per < 1200) ? 64 : 128;
     if (per < 1200) per_sm = 2;
@@ -330,7 +339,7 @@ static int coop_groups(long long ntotal, int num_sms) {
   return (g < 1) ? 1 : (g > 8) ? 8 : (int)g;
 }
 
-static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal, bool driver = false) {
+static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal, double dt, bool driver = false) {
   int b = h->p.block, per_sm = h->p.blocks_per_sm, lpc = h->p.lanes_per_cell;
   const bool coop_ok = (kmode == 1 || kmode == 2) && !batch;
   const tc_handle::Tuned& t = h->tuned[size_class(ntotal)];
@@ -349,7 +358,7 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal,
   if (lpc != 4) lpc = 1;
   if (auto_block) {
     int ps = 0;
-    default_block(kmode, ntotal, h->num_sms, b, ps);
+    default_block(kmode, ntotal, h->num_sms, dt, b, ps);
     // the drivers' plain iteration fills more warps (512,000 curve cells, ms at 2 / 4 blocks per
     // SM / the limit: 537 / 526 / 523; 300,000 slab cells 1262 / 1576 / 1906)
     if (driver_kernel(kmode, driver) && b == 128 && ps == 2) ps = 4;
@@ -430,7 +439,7 @@ static int enqueue(tc_handle* h, bool batch, const tcg::DevFields& f, long long 
   if (h->p.mode == TC_MODE_MIXED_SEEDED || h->p.mode == TC_MODE_NEWTON_FP64_SEEDED) {
     if (!h->d_mlp) return TC_ENOMLP;
   }
-  const Shape sh = launch_shape(h, kmode, batch, ntotal, driver);
+  const Shape sh = launch_shape(h, kmode, batch, ntotal, dt, driver);
   const int grid = sh.grid, block = sh.block;
   if (cudaMemsetAsync(h->d_cursor, 0, sizeof(unsigned long long), st) != cudaSuccess) return TC_ECUDA;
   tcg::DevParams dp = dev_params(h->p);
@@ -544,7 +553,7 @@ int tc_autotune(tc_handle* h, const tc_fields* f, double dt_s, void* stream, tc_
   h->p.lanes_per_cell = 0;
   rc = run(&ms0);
   const int reps = (rc == TC_OK && ms0 < 20.f) ? 3 : 1;
-  const Shape def = launch_shape(h, kmode, false, f->ncell);
+  const Shape def = launch_shape(h, kmode, false, f->ncell, dt_s);
   tc_tune_choice bestc = {0, 0, 0, 3.4e38f};
   auto candidate = [&](int block, int per_sm, int lpc) {
     h->p.block = block;
