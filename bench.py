@@ -45,12 +45,14 @@ FP64_NOMINAL_TFLOPS = 1.25
 STATE_KEYS = ("T", "xH2", "xHp")
 # DRAM bytes per cell of one k_step<1> launch on the 128^3 slab in the default shape (128
 # threads x 1216 blocks, 1024 resident threads per SM), from ncu (dram__bytes_read.sum +
-# dram__bytes_write.sum, one pass, profiles/step_counters.md): 13.49 GB read + 22.46 GB
+# dram__bytes_write.sum, one pass, profiles/step_counters.md): 13.21 GB read + 22.92 GB
 # written for 2,097,152 cells.  Almost all of it is the per-thread stack (spills at the
 # 64-register cap and the structs passed to the out-of-line physics), whose sum over the
-# resident threads exceeds L2.  The cells' own data are 152 B.
-TRAFFIC_BYTES_PER_CELL = 17145.0
-
+# resident threads exceeds L2, so it holds for that many threads and cells alone: a 64^3
+# launch of 128 x 152 moves 1.0 KB per cell.  The cells' own data are 152 B.
+TRAFFIC_BYTES_PER_CELL = 17228.0
+TRAFFIC_CELLS = 2097152
+TRAFFIC_SHAPE = {"block": (0, 128), "blocks_per_sm": (0, 8), "lanes_per_cell": (0, 1)}  # 0: the default
 
 def parse():
     ap = argparse.ArgumentParser()
@@ -641,9 +643,12 @@ def roofline_of(work, r, mode, ncell, peaks):
     fl = flops_per_cell(work[MODE_WORK[mode]], peaks["weights"]) * ncell
     achieved = fl / (r["kernel_ms"] * 1e-3) / 1e12
     peak = 2.0 * peaks["fp64_fma_per_s"] / 1e12
+    # the traffic figure is of one kernel in one shape on one grid
+    shape = r.get("launch_shape", {})
+    profiled = (mode == "newton" and ncell == TRAFFIC_CELLS and
+                all(shape.get(k, 0) in v for k, v in TRAFFIC_SHAPE.items()))
     return {"bound": "alu", "pipe": "fp64", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": achieved / peak, "traffic": (TRAFFIC_BYTES_PER_CELL * ncell
-                                           if mode == "newton" and TRAFFIC_BYTES_PER_CELL else None),
+            "frac": achieved / peak, "traffic": TRAFFIC_BYTES_PER_CELL * ncell if profiled else None,
             "peak_source": "measured FP64 FMA rate (library microbenchmark, this run); nominal %.2f" %
                            FP64_NOMINAL_TFLOPS,
             "work": "FP64 flops of the library's step per cell (work_slab128.json, %s) x %d cells" %
