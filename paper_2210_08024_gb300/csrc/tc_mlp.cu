@@ -352,6 +352,13 @@ int pass_grid(const tc_mlp* h, int B) {
   return (int)(tiles < h->num_sms ? tiles : h->num_sms);
 }
 
+// Whether n floats at a and m floats at b share memory.  The fused pass writes while other blocks
+// still read, so results that lie in their inputs go through a buffer.
+bool overlap(const float* a, size_t n, const float* b, size_t m) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+  return x < y + m * sizeof(float) && y < x + n * sizeof(float);
+}
+
 // splitmix64 (Steele, Lea & Flood 2014) for a reproducible weight initialisation.
 uint64_t splitmix64(uint64_t& s) {
   uint64_t z = (s += 0x9E3779B97F4A7C15ull);
@@ -456,21 +463,34 @@ int tc_mlp_get_params(const tc_mlp* h, float* theta) {
 int tc_mlp_predict(tc_mlp* h, const float* X, int B, float* out, void* stream) {
   if (!h || B < 0 || (B > 0 && (!X || !out))) return TC_EINVAL;
   if (B == 0) return TC_OK;
-  k_pass<false><<<pass_grid(h, B), NT, sizeof(Smem), (cudaStream_t)stream>>>(h->theta, h->norm, X, nullptr, B, 0.f, 0.f,
-                                                                             0.f, out, nullptr, nullptr, nullptr);
-  return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
+  cudaStream_t st = (cudaStream_t)stream;
+  const size_t n = (size_t)B * MLP_OUT;
+  float* o = out;
+  if (overlap(out, n, X, (size_t)B * MLP_IN) && cudaMallocAsync(&o, n * sizeof(float), st) != cudaSuccess) return TC_ENOMEM;
+  k_pass<false><<<pass_grid(h, B), NT, sizeof(Smem), st>>>(h->theta, h->norm, X, nullptr, B, 0.f, 0.f, 0.f, o, nullptr,
+                                                           nullptr, nullptr);
+  bool ok = cudaGetLastError() == cudaSuccess;
+  if (o != out) {
+    ok = cudaMemcpyAsync(out, o, n * sizeof(float), cudaMemcpyDeviceToDevice, st) == cudaSuccess && ok;
+    ok = cudaFreeAsync(o, st) == cudaSuccess && ok;
+  }
+  return ok ? TC_OK : TC_ECUDA;
 }
 
 int tc_mlp_grad(tc_mlp* h, const float* X, const float* Y, int B, const float* w3, float* grad, float* loss,
                 void* stream) {
   if (!h || B < 1 || !X || !Y) return TC_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  float* g = grad ? grad : h->grad;
+  const bool apart = grad && !overlap(grad, NPARAM, X, (size_t)B * MLP_IN) && !overlap(grad, NPARAM, Y, (size_t)B * MLP_OUT);
+  float* g = apart ? grad : h->grad;
   if (cudaMemsetAsync(g, 0, NPARAM * sizeof(float), st) != cudaSuccess) return TC_ECUDA;
   if (cudaMemsetAsync(h->acc, 0, sizeof(LossAcc), st) != cudaSuccess) return TC_ECUDA;
   const float w0 = w3 ? w3[0] : 1.f, w1 = w3 ? w3[1] : 1.f, w2 = w3 ? w3[2] : 1.f;
   k_pass<true><<<pass_grid(h, B), NT, sizeof(Smem), st>>>(h->theta, h->norm, X, Y, B, w0, w1, w2, nullptr, g, h->acc, loss);
-  return cudaGetLastError() == cudaSuccess ? TC_OK : TC_ECUDA;
+  if (cudaGetLastError() != cudaSuccess) return TC_ECUDA;
+  if (grad && !apart && cudaMemcpyAsync(grad, g, NPARAM * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+    return TC_ECUDA;
+  return TC_OK;
 }
 
 int tc_mlp_train_step(tc_mlp* h, const float* X, const float* Y, int B, const float* w3, float lr, float* loss,
