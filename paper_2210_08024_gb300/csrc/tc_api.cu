@@ -275,16 +275,16 @@ struct Shape {
 // Threads per block and resident blocks per SM (0: the occupancy limit) where neither the
 // caller nor the autotuner chose, one lane per cell, by the cells per SM.
 //  - Few cells take blocks of one warp: they spread over the SMs, and no lane waits for a
-//    block's other warps (random states by FP64 Newton, 32 / 128 threads: 4096 cells 49 / 61
-//    ms, 8000 46 / 58; 12,800 curve cells 15.1 / 15.7).
+//    block's other warps (random states by FP64 Newton, 32 / 128 threads: 4096 cells 27.8 / 31.5
+//    ms, 8000 33.0 / 36.5, 14,000 33.4 / 35.0).
 //  - FP64 modes: one warp per SM partition nearly fills its FP64 pipe (65 cycles an
 //    instruction, 77 with more), and fewer lanes take more cells each, longest first, so that
 //    lanes finish together.  More warps pay, by covering the rest, when each lane still gets
-//    a dozen cells.  ms at 4 / 8 / 16 warps per SM / the limit: slab by FP64 Newton 100k 7.0 /
-//    8.3 / 8.2 / 8.0, 300k 9.2 / 9.8 / 12.6 / 14.5, 600k 18.9 / 15.3 / 18.7 / 22.0, 1M 31.9 / 26.0
-//    / 26.1 / 30.2, 2M 67.6 / 55.0 / 55.3 / 51.7; by the paper's scheme 100k 3.0 / 4.2 / 5.4 / 5.5,
+//    a dozen cells.  ms at 4 / 8 / 16 warps per SM / the limit: slab by FP64 Newton 100k 5.4 /
+//    6.2 / 6.5 / 6.8, 300k 9.3 / 9.3 / 11.3 / 12.5, 600k 19.2 / 15.4 / 17.9 / 20.5, 1M 32.7 / 26.2
+//    / 26.2 / 29.1, 2M 66.6 / 52.6 / 52.5 / 49.6; by the paper's scheme 100k 3.0 / 4.2 / 5.4 / 5.5,
 //    300k 5.8 / 5.9 / 8.8 / 8.7, 885k 13.6 / 12.0 / 11.7 / 11.7; random states by FP64 Newton 30k
-//    58 / 67 / 72 / 66, 100k 113 / 97 / 128 / 147; seeded FP64 300k 33 / 43 / 54 / 57.
+//    38 / 46 / 45 / 47, 100k 74 / 65 / 91 / 101; seeded FP64 300k 33 / 43 / 54 / 57.
 //  - Mixed modes: large blocks run in step and fetch their code once (tc_kernels.cuh), which
 //    pays as soon as the cells fill them.  ms at 32 / 128 / 256 / 512 threads: seeded mixed, slab
 //    cells: 20k 5.4 / 5.5 / 5.8 / 6.4, 60k 6.8 / 6.4 / 6.6 / 6.6, 150k 10.3 / 9.3 / 8.3 / 9.2, 300k
@@ -318,8 +318,10 @@ static void default_block(int kmode, long long ntotal, int num_sms, double dt, i
 
 // Whether a launch of modes 1 and 2 takes four lanes per cell.
 //  - Mode 1: while the cells' warps of eight are at most two per SM partition, where latency
-//    decides (four and one lane agree to 1e-13).  ms with four / one: random states: 500 32 / 43,
-//    4096 37 / 49, 8000 44 / 46; slab: 8000 4.5 / 5.4.
+//    decides (four and one lane agree to 1e-13).  ms with four / one: random states: 500 20.4 /
+//    27.3, 2000 24.4 / 27.3, 4096 27.5 / 27.4, 8000 36.7 / 30.0; slab: 1000 over 100 yr 0.50 /
+//    0.64, 4800 over 1e3 yr 2.0 / 2.6, 8000 4.4 / 4.4.  (Drawn when more substeps took the plain
+//    iteration, which gains most by four lanes: 4096 37 / 49, 8000 44 / 46.)
 //  - Mode 2, and mode 1 by the drivers: while every cell's lanes are resident at once (19,456
 //    cells).  One lane is faster from 4864 cells on (random states: 8000 50 / 37; slab: 8000 4.8 /
 //    4.8; curve cells, mode 1: 12,800 62 / 57), but its results differ: in mode 2 by the polish's
@@ -396,8 +398,8 @@ static Shape launch_shape(tc_handle* h, int kmode, bool batch, long long ntotal,
 // over 1e3 yr 2.34 / 1.94, stiff cells 3.18 / 2.47, 1500 slab cells over 1e4 yr 3.61 / 3.26, 1000
 // over 100 yr 0.82 / 0.70, 4096 random states over 1e4 yr 36.2 / 30.9 (4800 over 100 yr 14.8 /
 // 16.2); mixed, 1500 slab cells over 1e4 yr 3.75 / 3.28, 4800 random states 32.3 / 33.9.  A cost
-// hint orders by the cost itself: alike cells then share a warp and its code (the PDR driver's
-// 48 x 100 cells 122 / 162 ms), so those and the drivers' first chunks stay with the queue, and so
+// hint orders by the cost itself: alike cells then share a warp and its code (48 x 100
+// PDR cells by these kernels 122 / 162 ms), so those and the drivers' first chunks stay with the queue, and so
 // do mixed launches of more than one warp per SM partition (16,000 cells, 1e4 yr: slab 4.96 / 7.02,
 // stiff 5.37 / 7.56, random states 65.5 / 72.8).
 static int dealt_cells(const Shape& sh, int kmode, long long ntotal, int num_sms) {

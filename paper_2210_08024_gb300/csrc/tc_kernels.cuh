@@ -101,8 +101,8 @@ TCG_FN float from_lane(float v, int r) {
 // (38 of them with the equilibrium's, 32 without): each lane evaluates every fourth one and
 // the values pass by shuffles, bit for bit those of chem_T and cool_T.  One warp a scheduler
 // issues an FP64 instruction every 65 cycles, whatever its lanes do, so the exponentials
-// were about a third of an evaluation's time.  1000 slab cells over 100 yr 526 -> 413 us, 48
-// PDR slabs of 100 cells over 30 chunks 134 -> 122 ms, 4096 random states 36.9 -> 35.4 ms.
+// were about a third of an evaluation's time.  1000 slab cells over 100 yr 526 -> 413 us,
+// 4096 random states 36.9 -> 35.4 ms.
 #ifdef __CUDACC__
 template <class FC>
 __device__ __noinline__ void temp_blocks_split(const CellC<FC>& c, double T, unsigned flags, bool eq, ChemT<double>& b,
@@ -636,7 +636,7 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 constexpr int TAN_MAXIT = 12;
 constexpr int TAN_MAXIT32 = 16;
 constexpr float TAN_STALE = 1e-2f;  // a Jacobian whose abundances were further off is rebuilt
-constexpr double TAN_TRACE = 1e-20;  // abundances below this take their step on their own, in FP64
+constexpr double TAN_TRACE = 1e-20;  // abundances below this are left to phase 2
 
 // source_tangents over the cell's lanes: with four, each takes one direction (the last
 // repeats the third) and they exchange.
@@ -818,7 +818,8 @@ TCG_FN int newton_tangent(const CellC<double>& c, const CellC<float>& cf, const 
     const float rtol = float(p.rtol);
     // how far this step's error can be from it: for the first step, from the Jacobian's
     // distance to the identity (relative units) and its error, 1e-3 of that at most (its
-    // FP32 rounding, and its change over phase 1's last step, 3e-5 times exponents up to 30)
+    // FP32 rounding, and its change over phase 1's last step, 3e-5 times exponents up to 30; where
+    // phase 1 ended at its floor up to 3e-2, and below 0.15 rtol remains)
     float left = (prev > 0.0f) ? rel / prev : 1.0f;
     if (it == 1) {
       float nj = 0.0f;
