@@ -291,11 +291,13 @@ struct Shape {
 //    14.8 / 11.8 / 10.5 / 10.5, 2M 44.4 (128) / 36.2 / 33.5; random states: 4k 40 / 44 / 50 / 62, 30k
 //    76 / 58 / 59 / 69, 100k 178 / 155 / 114 / 98.  At 100k one block of 256 an SM instead of
 //    the limit: slab seeded 7.2 -> 6.7, random states mixed 74 -> 62.
-//    Over short steps most cells take one substep, and seeded blocks of 256 mostly wait for the
-//    few that take more (ms with 256 (one an SM) / 128 / before the blocks met: stiff cells 100k
-//    over 100 yr 3.7 / 3.2 / 3.1, 300 yr 4.7 / 3.7 / 3.7, 1e3 yr 4.8 / 4.9 / 5.1; 160k over 100 yr
-//    4.2 / 3.9 / 3.9, 300 yr 4.7 / 4.5 / 4.9; slab cells over 100 yr, 170k 1.67 / 1.48 / 1.63).
-//    (Random states pay for it: 100k over 100 yr 40 / 64 / 95.)
+//    Over short steps most cells take one substep, and large blocks mostly wait for the few that
+//    take more.  Stiff cells, ms: seeded, 20k to 88k with 128 / 64 / before blocks met: 20k over
+//    300 yr 2.82 / 2.68 / 2.66, 1e3 yr 3.64 / 3.53 / 3.43, 60k over 1e3 yr 4.35 / 4.19 / 4.15; seeded,
+//    beyond with 256 (one an SM) / 128 / before: 100k over 100 yr 3.7 / 3.2 / 3.1, 300 yr 4.7 / 3.7 /
+//    3.7, 1e3 yr 4.8 / 4.9 / 5.1, 160k over 100 yr 4.2 / 3.9 / 3.9; mixed with 256 (one an SM) / 256
+//    to the limit / before: 100k over 100 yr 3.3 / 2.8 / 3.8, 300 yr 4.8 / 3.5 / 4.5.  Random states
+//    pay for it (seeded 30k over 100 yr 28 / 33 / 39, 100k 40 / 64 / 95; mixed 100k 35 / 39 / 100).
 constexpr double SHORT_STEP = 500.0 * 3.15576e7;
 static void default_block(int kmode, long long ntotal, int num_sms, double dt, int& b, int& per_sm) {
   const long long per = ntotal / num_sms;
@@ -304,9 +306,10 @@ static void default_block(int kmode, long long ntotal, int num_sms, double dt, i
     b = 32;
   } else if (kmode == 2 || kmode == 3) {
     b = (per < 600) ? 128 : (per < 1600) ? 256 : 512;
+    if (kmode == 3 && per < 600 && dt < 3.0 * SHORT_STEP) b = 64;
     if (b == 256 && per < 1200) {
-      if (kmode == 3 && dt < SHORT_STEP) b = 128;
-      else per_sm = 1;
+      if (dt >= SHORT_STEP) per_sm = 1;
+      else if (kmode == 3) b = 128;
     }
   } else {
     b = (per < 1200) ? 64 : 128;
