@@ -628,8 +628,8 @@ TCG_FN void start_sources(const CellC<F>& cf, const DevParams& p, const LaneStat
 //
 // `spent` receives the iterations of both phases.  Returns them, or -1 when a step would have to be damped, fails to
 // shrink by half or is not finite, or when TAN_MAXIT iterations pass; the plain solver then
-// takes the substep from its start, as if this one had not been tried.  Hard substeps (2% of
-// the random states' iterations, 0.04% of the slab's) thus keep the plain iteration's path,
+// takes the substep from its start, as if this one had not been tried.  Hard substeps (0.1% of
+// the random states', 0.004% of the slab's) thus keep the plain iteration's path,
 // with its damping, predictor and halving decisions.  (Damping here too solved some substeps
 // that the plain iteration halves, which changed the substep grid of 5 in 13,824 cells near
 // x_H = 0.)
